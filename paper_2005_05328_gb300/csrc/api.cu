@@ -96,7 +96,7 @@ struct Plan {
     cap = P.capacity ? (int64_t)P.capacity : (int64_t)P.n1d * P.n1d * P.n1d;
     node_cap = 2 * cap + 1024;
     m3 = (int64_t)P.mesh * P.mesh * P.mesh;
-    nspec = (int64_t)P.mesh * P.mesh * (P.mesh / 2 + 1);
+    nspec = (int64_t)P.mesh * P.mesh * (P.precision == DZS_FP64 ? spec_row<double>(P.mesh) : spec_row<float>(P.mesh));
     nb = (cap + 1023) / 1024;  // digit-histogram tiles: enough for sort tiles of >= 1024 keys
     nchunks = (cap + 1024) / 1024 + 1;
     ring = P.lc_capacity ? (int64_t)P.lc_capacity : cap;
@@ -139,7 +139,7 @@ struct Plan {
     o_phi = L.take(rsz * m3);
     o_cstart = L.take(4 * (m3 + 1));
     o_tw = L.take(2 * rsz * (P.mesh / 2 + 1));
-    o_green = L.take(rsz * (2 * P.mesh + 1));
+    o_green = L.take(rsz * (3 * P.mesh + 1));
     o_ring = L.take(sizeof(dzs_lc_record) * ring);
     o_n = L.take(16);
     o_err = L.take(16);

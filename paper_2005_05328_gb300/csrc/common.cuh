@@ -56,6 +56,18 @@ struct cplx {
   R x, y;
 };
 
+// mesh sizes whose transform takes three register stages (fft.cu), and the
+// row length of the half spectrum: those sizes pad the n/2 + 1 modes to 64
+// bytes
+template <class R>
+__host__ __device__ constexpr bool three_factor(int n) {
+  return sizeof(R) == 4 && (n == 256 || n == 512);
+}
+template <class R>
+__host__ __device__ constexpr int spec_row(int n) {
+  return three_factor<R>(n) ? (n / 2 + 8) & ~7 : n / 2 + 1;
+}
+
 template <class R>
 __device__ __forceinline__ cplx<R> cmul(cplx<R> a, cplx<R> b) {
   return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};

@@ -9,7 +9,8 @@
 //   X      -- same along ix; for the Poisson solve the forward FFT, the Green
 //             multiply and the inverse FFT are fused in one pass;
 //   Y inverse, Z c2r.
-// Each length-n transform is a four-step FFT, n = N1 N2 (n = 2^a, or 3 2^a
+// FP32 lengths 256 and 512 run as three register stages (k_fft3_*, below).
+// Every other length-n transform is a four-step FFT, n = N1 N2 (n = 2^a, or 3 2^a
 // with the factor 3 in N1; N2 a power of two): N2 register FFTs of length N1
 // (input stride N2; a length 3 M register FFT is three length-M FFTs and
 // radix-3 butterflies), twiddle W_n^(j2 k1),
@@ -336,6 +337,240 @@ __global__ void k_fft_cols(cplx<R>* __restrict__ spec, int W, int axis, int mode
   }
 }
 
+// ---- three-factor FP32 transforms of length 256 and 512 (n = 8 * 8 * n/64)
+//
+// A thread owns 8 elements of one column, T = n/8 threads share it: radix 8,
+// twiddle, exchange, radix 8, twiddle, exchange, radix 8 (512) or two radix 4
+// (256).  Bound by DRAM/L2 traffic: 16 data registers instead of the 64 a
+// two-factor split of 512 holds (32 complex; 130-157 registers, two blocks per
+// SM, half of its threads idle in the first half) keep 3-4 times the loads in
+// flight, and every thread works in every stage.  Rows of the half spectrum
+// are padded to 64 bytes so that 8 consecutive columns are two whole sectors.
+// Each transform leaves thread u with the elements u + T j, the distribution
+// it began with, so that the X pass runs forward, Green multiply and inverse
+// without a trip through memory.  Measured, the five passes of the Poisson
+// solve: 512^3 4.05 -> 1.73 ms (Z passes 1.34 -> 0.32 and 1.4 -> 0.29, Y 0.43
+// -> 0.27, X with the Green factor 0.57: 1.9-3.8 TB/s of 6.8), 256^3 0.284 ->
+// 0.218 ms.  At 128 and below, and in FP64, a two-factor transform already
+// holds at most 16 elements a thread and stays.
+// Shared slots of a column: [8][kSA] after the first stage, [8][kSB] after
+// the second with rows of 9: at one column per group of threads (Z) and at 8
+// interleaved columns (Y, X) the lanes of a half warp fall on distinct banks
+// (but for a few pairs of the 256-point Z transform).
+template <int N>
+struct Tri {
+  static constexpr int T = N / 8, R2 = N / 64;
+  static constexpr int kSA = T + R2, kSB = R2 * 9 + 1;
+  static constexpr int kSlots = 8 * (kSB > kSA ? kSB : kSA);
+};
+
+__device__ __forceinline__ cplx<float> cadd(cplx<float> a, cplx<float> b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ cplx<float> csub(cplx<float> a, cplx<float> b) { return {a.x - b.x, a.y - b.y}; }
+// times -i (forward) or i (inverse)
+template <bool kInv>
+__device__ __forceinline__ cplx<float> cquarter(cplx<float> a) {
+  return kInv ? cplx<float>{-a.y, a.x} : cplx<float>{a.y, -a.x};
+}
+
+template <bool kInv>
+__device__ __forceinline__ void fft4(cplx<float>& a0, cplx<float>& a1, cplx<float>& a2, cplx<float>& a3) {
+  const cplx<float> s0 = cadd(a0, a2), d0 = csub(a0, a2), s1 = cadd(a1, a3), d1 = cquarter<kInv>(csub(a1, a3));
+  a0 = cadd(s0, s1);
+  a1 = cadd(d0, d1);
+  a2 = csub(s0, s1);
+  a3 = csub(d0, d1);
+}
+
+template <bool kInv>
+__device__ __forceinline__ void fft8(cplx<float> (&a)[8]) {
+  constexpr float h = 0.70710678118654752f;
+  cplx<float> e0 = cadd(a[0], a[4]), e1 = cadd(a[1], a[5]), e2 = cadd(a[2], a[6]), e3 = cadd(a[3], a[7]);
+  cplx<float> o0 = csub(a[0], a[4]), o1 = csub(a[1], a[5]), o2 = cquarter<kInv>(csub(a[2], a[6])),
+              o3 = csub(a[3], a[7]);
+  // odd half times exp(-+ 2 pi i j / 8)
+  o1 = kInv ? cplx<float>{h * (o1.x - o1.y), h * (o1.x + o1.y)} : cplx<float>{h * (o1.x + o1.y), h * (o1.y - o1.x)};
+  o3 = kInv ? cplx<float>{-h * (o3.x + o3.y), h * (o3.x - o3.y)} : cplx<float>{h * (o3.y - o3.x), -h * (o3.x + o3.y)};
+  fft4<kInv>(e0, e1, e2, e3);
+  fft4<kInv>(o0, o1, o2, o3);
+  a[0] = e0;
+  a[1] = o0;
+  a[2] = e1;
+  a[3] = o1;
+  a[4] = e2;
+  a[5] = o2;
+  a[6] = e3;
+  a[7] = o3;
+}
+
+// one column: thread u (< T) enters with the elements u + T j in a[j] and
+// leaves with the transform's elements u + T j; at(slot) is the column's
+// shared-memory slot.  Every thread of the block calls it (block barriers);
+// the buffer is free for reuse after the next barrier.
+template <int N, bool kInv, class At>
+__device__ __forceinline__ void tri_fft(cplx<float> (&a)[8], cplx<float>* buf, At at, int u,
+                                        const cplx<float>* __restrict__ tw) {
+  using S = Tri<N>;
+  fft8<kInv>(a);
+#pragma unroll
+  for (int k = 1; k < 8; ++k) a[k] = cmul(a[k], twn(tw, u * k, N, kInv));
+#pragma unroll
+  for (int k = 0; k < 8; ++k) buf[at(k * S::kSA + u)] = a[k];
+  __syncthreads();
+  const int t1 = u % S::R2, q0 = u / S::R2;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) a[j] = buf[at(q0 * S::kSA + t1 + S::R2 * j)];
+  fft8<kInv>(a);
+#pragma unroll
+  for (int k = 1; k < 8; ++k) a[k] = cmul(a[k], twn(tw, 8 * t1 * k, N, kInv));
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) buf[at(q0 * S::kSB + t1 * 9 + k)] = a[k];
+  __syncthreads();
+  const int p0 = (u & 7) * S::kSB, p1 = u >> 3;
+  if (S::R2 == 8) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) a[j] = buf[at(p0 + j * 9 + p1)];
+    fft8<kInv>(a);
+  } else {
+    // two groups of four: elements u + T (g + 2 k)
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) a[g + 2 * j] = buf[at(p0 + j * 9 + p1 + 4 * g)];
+    }
+    fft4<kInv>(a[0], a[2], a[4], a[6]);
+    fft4<kInv>(a[1], a[3], a[5], a[7]);
+  }
+}
+
+constexpr int kTriCols = 8;       // columns of a Y or X block (64 bytes of each row)
+constexpr int kTriThreads = 256;  // threads of a Z block: kTriThreads / T row pairs
+
+template <int N>
+__global__ void __launch_bounds__(kTriThreads) k_fft3_z_r2c(const float* __restrict__ in,
+                                                            cplx<float>* __restrict__ out,
+                                                            const cplx<float>* __restrict__ tw) {
+  using S = Tri<N>;
+  constexpr int T = S::T, HP = spec_row<float>(N);
+  __shared__ cplx<float> sm[kTriThreads / T][S::kSlots];
+  const int u = threadIdx.x % T, w = threadIdx.x / T;
+  const int64_t pr = (int64_t)blockIdx.x * (kTriThreads / T) + w;  // N^2 / 2 pairs: a multiple of the block's
+  cplx<float>* buf = sm[w];
+  const float *r0 = in + 2 * pr * N, *r1 = r0 + N;
+  cplx<float> a[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) a[j] = {r0[u + T * j], r1[u + T * j]};
+  tri_fft<N, false>(a, buf, [](int s) { return s; }, u, tw);
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < 8; ++j) buf[u + T * j] = a[j];
+  __syncthreads();
+  // X_a = (Z_k + conj Z_-k) / 2,  X_b = (Z_k - conj Z_-k) / (2 i)
+  cplx<float>*o0 = out + 2 * pr * HP, *o1 = o0 + HP;
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    if (j == 4 && u != 0) break;
+    const int k = u + T * j;
+    const cplx<float> z = a[j], zc = buf[(N - k) & (N - 1)];
+    o0[k] = {0.5f * (z.x + zc.x), 0.5f * (z.y - zc.y)};
+    o1[k] = {0.5f * (z.y + zc.y), -0.5f * (z.x - zc.x)};
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(kTriThreads) k_fft3_z_c2r(const cplx<float>* __restrict__ in,
+                                                            float* __restrict__ out,
+                                                            const cplx<float>* __restrict__ tw) {
+  using S = Tri<N>;
+  constexpr int T = S::T, HP = spec_row<float>(N);
+  __shared__ cplx<float> sm[kTriThreads / T][S::kSlots];
+  const int u = threadIdx.x % T, w = threadIdx.x / T;
+  const int64_t pr = (int64_t)blockIdx.x * (kTriThreads / T) + w;
+  cplx<float>* buf = sm[w];
+  const cplx<float>*i0 = in + 2 * pr * HP, *i1 = i0 + HP;
+  cplx<float> a[8];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    if (j == 4 && u != 0) break;
+    const int k = u + T * j;
+    const cplx<float> p = i0[k], q = i1[k];
+    a[j] = {p.x - q.y, p.y + q.x};               // Z_k = A_k + i B_k
+    const int m = (N - k) & (N - 1);             // Z_-k = conj A_k + i conj B_k
+    if (m >= N / 2) buf[m] = j == 4 ? a[j] : cplx<float>{p.x + q.y, q.x - p.y};
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 4; j < 8; ++j) a[j] = buf[u + T * j];
+  __syncthreads();
+  tri_fft<N, true>(a, buf, [](int s) { return s; }, u, tw);
+  float *r0 = out + 2 * pr * N, *r1 = r0 + N;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    r0[u + T * j] = a[j].x;
+    r1[u + T * j] = a[j].y;
+  }
+}
+
+// Y (axis 1) or X (axis 0) pass, modes as k_fft_cols.  The Green factor is
+// gfac / k^2 times one precomputed exp(-k_i^2 r_s^2) / W(k_i)^2 per axis.
+template <int N, int kMode>
+__global__ void __launch_bounds__(Tri<N>::T* kTriCols, 1024 / (Tri<N>::T * kTriCols))
+    k_fft3_cols(cplx<float>* __restrict__ spec, int axis, const cplx<float>* __restrict__ tw,
+                const float* __restrict__ gtab, float gfac) {
+  using S = Tri<N>;
+  constexpr int T = S::T, HN = N / 2 + 1, HP = spec_row<float>(N), W = kTriCols;
+  __shared__ cplx<float> buf[S::kSlots * W];
+  constexpr int ncb = (HN + W - 1) / W;
+  const int line = blockIdx.x / ncb;
+  const int col = threadIdx.x % W, u = threadIdx.x / W, kz = (blockIdx.x % ncb) * W + col;
+  const int64_t es = axis == 1 ? (int64_t)HP : (int64_t)N * HP;
+  cplx<float>* base = spec + (axis == 1 ? (int64_t)line * N * HP : (int64_t)line * HP) + kz;
+  const bool valid = kz < HN;
+  cplx<float> a[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) a[j] = valid ? base[(u + T * j) * es] : cplx<float>{0.f, 0.f};
+  auto at = [col](int s) { return s * W + col; };
+  tri_fft<N, kMode == 1>(a, buf, at, u, tw);
+  if (kMode == 2) {
+    const float *k2t = gtab, *et = gtab + 2 * N + 1;
+    const float k2l = valid ? k2t[line] + k2t[kz] : 0.f, el = valid ? gfac * et[line] * et[kz] : 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float kk = k2t[u + T * j] + k2l;
+      const float gv = kk > 0.f ? el * et[u + T * j] / kk : 0.f;
+      a[j] = {a[j].x * gv, a[j].y * gv};
+    }
+    __syncthreads();
+    tri_fft<N, true>(a, buf, at, u, tw);
+  }
+  if (!valid) return;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) base[(u + T * j) * es] = a[j];
+}
+
+template <int N>
+void launch3_r2c_zy(dzs_ctx* c, const float* in, cplx<float>* out, const cplx<float>* tw, bool do_x) {
+  using S = Tri<N>;
+  const unsigned zb = (unsigned)((int64_t)N * N / 2 / (kTriThreads / S::T));
+  const unsigned cb = N * ((N / 2 + 1 + kTriCols - 1) / kTriCols);
+  k_fft3_z_r2c<N><<<zb, kTriThreads, 0, c->stream>>>(in, out, tw);
+  k_fft3_cols<N, 0><<<cb, S::T * kTriCols, 0, c->stream>>>(out, 1, tw, nullptr, 0.f);
+  if (do_x) k_fft3_cols<N, 0><<<cb, S::T * kTriCols, 0, c->stream>>>(out, 0, tw, nullptr, 0.f);
+}
+
+template <int N>
+void launch3_c2r(dzs_ctx* c, cplx<float>* in, float* out, const cplx<float>* tw, const float* green, float gfac) {
+  using S = Tri<N>;
+  const unsigned zb = (unsigned)((int64_t)N * N / 2 / (kTriThreads / S::T));
+  const unsigned cb = N * ((N / 2 + 1 + kTriCols - 1) / kTriCols);
+  if (green)
+    k_fft3_cols<N, 2><<<cb, S::T * kTriCols, 0, c->stream>>>(in, 0, tw, green, gfac);
+  else
+    k_fft3_cols<N, 1><<<cb, S::T * kTriCols, 0, c->stream>>>(in, 0, tw, nullptr, 0.f);
+  k_fft3_cols<N, 1><<<cb, S::T * kTriCols, 0, c->stream>>>(in, 1, tw, nullptr, 0.f);
+  k_fft3_z_c2r<N><<<zb, kTriThreads, 0, c->stream>>>(in, out, tw);
+}
+
 template <class R, int N>
 int cols_per_block() {
   // W * N1 threads per block, at most 256; shared memory srows(W) * N * sizeof(cplx)
@@ -346,26 +581,36 @@ int cols_per_block() {
 
 template <class R, int N>
 void launch_r2c_zy(dzs_ctx* c, const R* in, cplx<R>* out, const cplx<R>* tw, bool do_x) {
-  const int W = cols_per_block<R, N>();
-  const int threads = W * Split<N>::N1;
-  const size_t sm = (size_t)N * srows(W) * sizeof(cplx<R>);
-  const int64_t npairs = (int64_t)N * N / 2;
-  k_fft_z_r2c<R, N><<<(unsigned)((npairs + W - 1) / W), threads, sm, c->stream>>>(in, out, W, npairs, tw);
-  const int ncb = (N / 2 + 1 + W - 1) / W;
-  k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(out, W, 1, 0, tw, nullptr, (R)0);
-  if (do_x) k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(out, W, 0, 0, tw, nullptr, (R)0);
+  if constexpr (three_factor<R>(N)) {
+    launch3_r2c_zy<N>(c, in, out, tw, do_x);
+    return;
+  } else {
+    const int W = cols_per_block<R, N>();
+    const int threads = W * Split<N>::N1;
+    const size_t sm = (size_t)N * srows(W) * sizeof(cplx<R>);
+    const int64_t npairs = (int64_t)N * N / 2;
+    k_fft_z_r2c<R, N><<<(unsigned)((npairs + W - 1) / W), threads, sm, c->stream>>>(in, out, W, npairs, tw);
+    const int ncb = (N / 2 + 1 + W - 1) / W;
+    k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(out, W, 1, 0, tw, nullptr, (R)0);
+    if (do_x) k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(out, W, 0, 0, tw, nullptr, (R)0);
+  }
 }
 
 template <class R, int N>
 void launch_c2r(dzs_ctx* c, cplx<R>* in, R* out, const cplx<R>* tw, const R* green, R gfac) {
-  const int W = cols_per_block<R, N>();
-  const int threads = W * Split<N>::N1;
-  const size_t sm = (size_t)N * srows(W) * sizeof(cplx<R>);
-  const int64_t npairs = (int64_t)N * N / 2;
-  const int ncb = (N / 2 + 1 + W - 1) / W;
-  k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(in, W, 0, green ? 2 : 1, tw, green, gfac);
-  k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(in, W, 1, 1, tw, nullptr, (R)0);
-  k_fft_z_c2r<R, N><<<(unsigned)((npairs + W - 1) / W), threads, sm, c->stream>>>(in, out, W, npairs, tw);
+  if constexpr (three_factor<R>(N)) {
+    launch3_c2r<N>(c, in, out, tw, green, gfac);
+    return;
+  } else {
+    const int W = cols_per_block<R, N>();
+    const int threads = W * Split<N>::N1;
+    const size_t sm = (size_t)N * srows(W) * sizeof(cplx<R>);
+    const int64_t npairs = (int64_t)N * N / 2;
+    const int ncb = (N / 2 + 1 + W - 1) / W;
+    k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(in, W, 0, green ? 2 : 1, tw, green, gfac);
+    k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(in, W, 1, 1, tw, nullptr, (R)0);
+    k_fft_z_c2r<R, N><<<(unsigned)((npairs + W - 1) / W), threads, sm, c->stream>>>(in, out, W, npairs, tw);
+  }
 }
 
 template <class R>

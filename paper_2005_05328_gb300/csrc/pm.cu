@@ -445,7 +445,7 @@ template <class R>
 __global__ void k_pk_plane(const cplx<R>* __restrict__ spec, int M, const R* __restrict__ gtab, int nbins,
                            double norm, double shot, double kf, double* __restrict__ part) {
   extern __shared__ double wrow[];  // [warps][nbins][3]: modes, sum |k|, sum P
-  const int kx = blockIdx.x, HN = M / 2 + 1;
+  const int kx = blockIdx.x, HN = M / 2 + 1, HP = spec_row<R>(M);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int q = threadIdx.x; q < nw * nbins * 3; q += blockDim.x) wrow[q] = 0.0;
   __syncthreads();
@@ -462,7 +462,7 @@ __global__ void k_pk_plane(const cplx<R>* __restrict__ spec, int M, const R* __r
       const int64_t n2 = (int64_t)sx * sx + (int64_t)sy * sy + (int64_t)kz * kz;
       b = mode_bin(n2);
       if (b >= 1 && b <= nbins) {
-        const cplx<R> d = spec[((int64_t)kx * M + ky) * HN + kz];
+        const cplx<R> d = spec[((int64_t)kx * M + ky) * HP + kz];
         const double wv = (double)wt[kx] * (double)wt[ky] * (double)wt[kz];
         const double p = ((double)d.x * (double)d.x + (double)d.y * (double)d.y) * norm / (wv * wv) - shot;
         cnt = (kz == 0 || 2 * kz == M) ? 1.0 : 2.0;
@@ -593,7 +593,8 @@ void launch_pm_interp(dzs_ctx* c) {
 template <class R>
 std::vector<cplx<R>> twiddles(int n);
 
-// twiddles of size M and the per-axis Green tables (k^2, W_CIC, r_s^2)
+// twiddles of size M and the per-axis Green tables: k^2, W_CIC, r_s^2, and
+// exp(-k^2 r_s^2) / W_CIC^2
 void launch_fft_init(dzs_ctx* c) {
   upload_fft_constants(c->dev);
   const int M = c->M;
@@ -610,20 +611,22 @@ void launch_fft_init(dzs_ctx* c) {
   if (c->fp64) {
     auto tw = twiddles<double>(M);
     cudaMemcpy(c->B.twiddle, tw.data(), tw.size() * sizeof(cplx<double>), cudaMemcpyHostToDevice);
-    std::vector<double> g(2 * M + 1);
+    std::vector<double> g(3 * M + 1);
     for (int m = 0; m < M; ++m) {
       g[m] = k2[m];
       g[M + m] = w[m];
+      g[2 * M + 1 + m] = std::exp(-k2[m] * rs2) / (w[m] * w[m]);
     }
     g[2 * M] = rs2;
     cudaMemcpy(c->B.green_axis, g.data(), g.size() * sizeof(double), cudaMemcpyHostToDevice);
   } else {
     auto tw = twiddles<float>(M);
     cudaMemcpy(c->B.twiddle, tw.data(), tw.size() * sizeof(cplx<float>), cudaMemcpyHostToDevice);
-    std::vector<float> g(2 * M + 1);
+    std::vector<float> g(3 * M + 1);
     for (int m = 0; m < M; ++m) {
       g[m] = (float)k2[m];
       g[M + m] = (float)w[m];
+      g[2 * M + 1 + m] = (float)(std::exp(-k2[m] * rs2) / (w[m] * w[m]));
     }
     g[2 * M] = (float)rs2;
     cudaMemcpy(c->B.green_axis, g.data(), g.size() * sizeof(float), cudaMemcpyHostToDevice);
