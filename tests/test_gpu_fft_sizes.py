@@ -55,3 +55,30 @@ def test_potential_matches_fp64_fft(dzs, precision, mesh):
     tol = 8e-7 if precision == 0 else 8e-7 * 2.0 ** -29
     assert math.sqrt((err ** 2).mean()) <= tol * rms
     assert err.max() <= 6 * tol * max(rms, np.abs(want).max())
+
+
+@pytest.mark.parametrize("mesh,nbins", [(8, 1), (8, 4), (16, 7), (24, 12), (32, 16), (96, 41), (256, 128)])
+def test_power_spectrum_bins(dzs, mesh, nbins):
+    """Counts exact, mean |k| to FP64 rounding, P(k) of a random set against
+    numpy sums over the same modes (FP64 contexts: 1e-12 of the bin's power;
+    the small meshes cover one split per plane and rows shorter than a warp)"""
+    n1d, box = 16, 32.0
+    rng = np.random.default_rng(mesh + nbins)
+    n = n1d ** 3
+    st = dict(u=rng.integers(0, 2 ** 32, size=(3, n), dtype=np.uint64).astype(np.uint32), p=np.zeros((3, n)),
+              g=np.zeros((3, n)), k=np.ones(n, np.uint32), id=np.arange(n, dtype=np.uint32), fl=np.zeros(n, np.uint8))
+    with dzs.Context(n1d=n1d, mesh=mesh, box=box, precision=1, dzs_on=0) as ctx:
+        ctx.set_state(st, 0)
+        k, pk, modes = ctx.power_spectrum(nbins, shot=False)
+        delta = ctx.mesh(dzs.MESH_DELTA)
+    f = np.fft.fftfreq(mesh, 1.0 / mesh)
+    n2 = f[:, None, None] ** 2 + f[None, :, None] ** 2 + f[None, None, :] ** 2
+    w = np.sinc(f / mesh) ** 2
+    power = np.abs(np.fft.fftn(delta)) ** 2 * (box / mesh ** 2) ** 3 / (
+        w[:, None, None] * w[None, :, None] * w[None, None, :]) ** 2
+    b = np.floor(np.sqrt(n2) + 0.5).astype(int)
+    for q in range(1, nbins + 1):
+        sel = b == q
+        assert modes[q - 1] == sel.sum()
+        assert k[q - 1] == pytest.approx(2 * math.pi / box * np.sqrt(n2[sel]).mean(), rel=1e-13)
+        assert pk[q - 1] == pytest.approx(power[sel].mean(), rel=1e-12)
