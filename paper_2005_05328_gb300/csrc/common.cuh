@@ -255,6 +255,7 @@ void launch_mass_prefix(dzs_ctx* c);
 void launch_amin2(dzs_ctx* c);
 void launch_tree(dzs_ctx* c);
 void launch_cell_start(dzs_ctx* c);
+void launch_cells(dzs_ctx* c, int depth);
 void launch_pm_deposit(dzs_ctx* c);
 void launch_pm_fft(dzs_ctx* c);
 void launch_pm_interp(dzs_ctx* c);

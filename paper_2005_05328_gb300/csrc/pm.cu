@@ -623,13 +623,16 @@ void launch_sum_k2(dzs_ctx* c, unsigned long long* out) {
 // the PM force in three stages: CIC deposit of delta; FFT Poisson solve with
 // the Green function fused into the X pass (phi); four-point gradient and
 // CIC interpolation to the particles (g)
-// CSR table of the depth-m Morton cells (m = log2 M) of the current keys
-void launch_cell_start(dzs_ctx* c) {
+// CSR table of the Morton cells of a depth of the current keys
+void launch_cells(dzs_ctx* c, int depth) {
   c->launches += 1;
-  const int64_t ncell = (int64_t)1 << (3 * c->logM);  // M^3 for M = 2^m
-  const int sh = 3 * (kMaxLevel - c->logM);
+  const int64_t ncell = (int64_t)1 << (3 * depth);
+  const int sh = 3 * (kMaxLevel - depth);
   k_cell_start<<<grid_for(c->N0 + 1), kThreads, 0, c->stream>>>(c->B.n, c->B.key, sh, ncell, c->B.cell_start);
 }
+
+// depth m = log2 M: the mesh cells of M = 2^m
+void launch_cell_start(dzs_ctx* c) { launch_cells(c, c->logM); }
 
 void launch_pm_deposit(dzs_ctx* c) {
   c->launches += c->mesh_pow2 ? 2 : 16;
