@@ -433,6 +433,7 @@ dzs_status dzs_create(const dzs_params* p, void* cuda_stream, dzs_ctx** out) {
     return fail(nullptr, DZS_ECUDA, "arena init");
   }
   launch_fft_init(c);
+  if (c->fp64 && !upload_walk_constants(c->dev)) st = DZS_ECUDA;
   if (cudaDeviceSynchronize() != cudaSuccess) st = DZS_ECUDA;
   if (st != DZS_OK) {
     cudaFree(c->arena);

@@ -260,6 +260,7 @@ void launch_pm_deposit(dzs_ctx* c);
 void launch_pm_fft(dzs_ctx* c);
 void launch_pm_interp(dzs_ctx* c);
 void launch_walk(dzs_ctx* c, bool tree, bool close_kick, int step);
+bool upload_walk_constants(int dev);  // the FP64 pair table, once per device
 void launch_diagnostics(dzs_ctx* c);
 void launch_ics(dzs_ctx* c);
 void launch_to_double(dzs_ctx* c, const void* src, int64_t count, double* dst);

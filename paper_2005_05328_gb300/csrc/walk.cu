@@ -45,9 +45,11 @@
 // fixed shuffle tree (the result is deterministic).  Pair force: softened
 // 1/r^3 times T(r) = erfc(x) + (2/sqrt(pi)) x exp(-x^2), x = r / 2 r_s, zero
 // at r = 0 and r >= r_cut.  FP32 evaluates T = exp(-x^2) Q(x) with a fitted
-// polynomial (gen_split_poly.py, relative error 3.3e-7); FP64 calls erfc and
-// exp.
+// polynomial (gen_split_poly.py, relative error 3.3e-7); FP64 reads T(r) / r^3
+// from a table of polynomials in r^2.
 #include <cmath>
+#include <mutex>
+#include <vector>
 
 #include "common.cuh"
 
@@ -149,6 +151,20 @@ struct WalkSmem {
   R h[kWarps][kList];  // spline radius 2.8 eps of the entry (lattice units)
 };
 
+// FP64 pair factor: F(z) = T(sqrt z) z^(-3/2), z = (r / 2 r_s)^2, so that
+// T(r) / r^3 = F / (2 r_s)^3 needs no square root, division, erfc or exp.
+// FP64 runs 2 multiply-adds per clock and SM, and those four took ~100 of
+// them; a degree-7 polynomial per 1/64 octave of z (Chebyshev interpolation,
+// truncated below 1e-17 relative; 1/32 octave leaves 2e-15 at z > 4) takes 7.
+// z outside the table (2^-12 .. 2^3; r_cut = 4.5 r_s is z = 5.06) and softened
+// pairs take the formula.  60 KB, of which the usual z in [0.3, 5] touch 16,
+// read through L1.  With range tests in FP32, walk of 32^3 / mesh 64 early in a
+// run 2.05 -> 0.40 ms, of 64^3 / mesh 128 10.7 -> 1.86 ms; forces 2e-16 (2-norm)
+// from the formula's.
+constexpr int kZSub = 64, kZDeg = 7, kZLo = -12, kZHi = 3;
+constexpr int kZCells = (kZHi - kZLo) * kZSub;
+__device__ __align__(64) double kZTab[kZCells][kZDeg + 1];
+
 // everything in lattice units (s = L / 2^32): a = sum (G m / s^2) X fac(R) T(s R)
 template <class R>
 struct WalkConst {
@@ -156,7 +172,10 @@ struct WalkConst {
   R inv2rs;  // s / (2 r_s)
   R tcoef;   // (s / 2 r_s) * 2 / x_max (polynomial variable t = r tcoef - 1)
   R nl2;     // -log2(e) (s / 2 r_s)^2
-  R gm0;     // G m0 / s^2
+  R gm0;     // G m0 / s^2 (FP64: times (s / 2 r_s)^3, the scale of F)
+  R zscale;  // FP64: (s / 2 r_s)^2
+  R igscale; // FP64: (2 r_s / s)^3
+  float rcut2_hi;  // FP64: FP32 bound above r_cut^2 (relative margin 2^-20)
   R kick;    // closing kick factor
   uint64_t skip_d2;                 // not skipped iff cube gap^2 <= skip_d2
   uint64_t open_d2[kMaxLevel + 1];  // opened iff COM distance^2 <= open_d2[level]
@@ -232,10 +251,6 @@ __device__ __forceinline__ void inv_and_r(float r2, float& r, float& ir) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(r2));
   r = r2 * ir;
 }
-__device__ __forceinline__ void inv_and_r(double r2, double& r, double& ir) {
-  r = sqrt(r2);
-  ir = 1.0 / r;
-}
 
 // squared lattice distance of entry E from the lane's particle P: FP32 from
 // the two offsets from the group centre, FP64 from the exact int32
@@ -262,67 +277,107 @@ __device__ __forceinline__ bool in_range(float r2, float rcut2) {
 }
 __device__ __forceinline__ bool in_range(double r2, double rcut2) { return r2 < rcut2 && r2 > 0.0; }
 
-// force of one entry at offset (dx, dy, dz), 0 < r^2 < r_cut^2 (the caller
-// has tested the range)
-template <class R>
-__device__ __forceinline__ void pair_force(R dx, R dy, R dz, R r2, R m, const R* hep, R hi, R hmax,
-                                           const WalkConst<R>& C, R& ax, R& ay, R& az) {
-  R r, ir;
-  inv_and_r(r2, r, ir);
-  R fac = ir * ir * ir;
-  // the entry's spline radius is read only when some softening of this step
-  // reaches r (hmax: the largest radius of any particle or node)
-  if (r < hmax) {
-    const R he = *hep, h = he > hi ? he : hi;
-    if (r < h) {
-      if (sizeof(R) == 4)
-        fac = (R)spline_fac_ir((float)r, (float)ir, (float)h);
-      else
-        fac = spline_fac(r, h);
+// FP64: FP32 squared distance bounds the range from above (its error is below
+// 2^-21 relative; 0 exactly for the self pair), so that only pairs in range, and
+// a rare one at its edge, reach the FP64 unit
+__device__ __forceinline__ bool maybe_in_range(const LEntry<double>& E, const Pos<double>& P, float rcut2_hi) {
+  const float dx = (float)(int32_t)(E.x - P.x), dy = (float)(int32_t)(E.y - P.y), dz = (float)(int32_t)(E.z - P.z);
+  return in_range(fmaf(dx, dx, fmaf(dy, dy, dz * dz)), rcut2_hi);
+}
+
+// one pair of FP64 entries: exact range test, then the table (or, softened or
+// outside it, the formula)
+__device__ __forceinline__ void pair_fp64(const LEntry<double>& E, const double* hep, const Pos<double>& P, double hi,
+                                          double hmax, const WalkConst<double>& C, double& ax, double& ay, double& az,
+                                          unsigned& nin) {
+  double dx, dy, dz;
+  const double r2 = entry_r2(E, P, dx, dy, dz);
+  if (!in_range(r2, C.rcut2)) return;
+  ++nin;
+  const double z = r2 * C.zscale;
+  const int cell = (int)(__double2hiint(z) >> 14) - ((1023 + kZLo) << 6);  // exponent and 6 mantissa bits
+  double f = 0.0;
+  bool done = false;
+  if (r2 < hmax * hmax) {
+    const double he = *hep, h = he > hi ? he : hi;
+    if (r2 < h * h) {
+      const double r = sqrt(r2);
+      f = C.igscale * spline_fac(r, h) * split_factor(r * C.inv2rs, 0);
+      done = true;
     }
   }
-  R sfac;
-  if (sizeof(R) == 4 && C.poly) {
-    const float t = fmaf((float)r, (float)C.tcoef, -1.0f);
-    float q = kSplitPoly[11];
-#pragma unroll
-    for (int i = 10; i >= 0; --i) q = fmaf(q, t, kSplitPoly[i]);
-    sfac = (R)(ex2_approx((float)r2 * (float)C.nl2) * q);
-  } else {
-    sfac = split_factor(r * C.inv2rs, C.poly);
+  if (!done) {
+    if (cell >= 0 && cell < kZCells) {
+      // the middle of the cell: the 46 low mantissa bits replaced by 1000...
+      const double t = z - __hiloint2double((__double2hiint(z) & ~0x3fff) | 0x2000, 0);
+      const double2* q = reinterpret_cast<const double2*>(kZTab[cell]);
+      const double2 q3 = q[3], q2 = q[2], q1 = q[1], q0 = q[0];
+      f = fma(q3.y, t, q3.x);
+      f = fma(f, t, q2.y);
+      f = fma(f, t, q2.x);
+      f = fma(f, t, q1.y);
+      f = fma(f, t, q1.x);
+      f = fma(f, t, q0.y);
+      f = fma(f, t, q0.x);
+    } else {
+      const double r = sqrt(r2);
+      f = C.igscale * split_factor(r * C.inv2rs, 0) / (r2 * r);
+    }
   }
-  const R f = m * fac * sfac;
+  f *= E.m;
   ax += f * dx;
   ay += f * dy;
   az += f * dz;
 }
 
-template <class R>
-__device__ __forceinline__ void pair_in_range(const LEntry<R>& E, const R* hep, const Pos<R>& P, R hi, R hmax,
-                                              const WalkConst<R>& C, R& ax, R& ay, R& az) {
-  R dx, dy, dz;
-  const R r2 = entry_r2(E, P, dx, dy, dz);
-  pair_force(dx, dy, dz, r2, E.m, hep, hi, hmax, C, ax, ay, az);
+// force of one FP32 entry at offset (dx, dy, dz), 0 < r^2 < r_cut^2 (the caller
+// has tested the range)
+__device__ __forceinline__ void pair_force(float dx, float dy, float dz, float r2, float m, const float* hep, float hi,
+                                           float hmax, const WalkConst<float>& C, float& ax, float& ay, float& az) {
+  float r, ir;
+  inv_and_r(r2, r, ir);
+  float fac = ir * ir * ir;
+  // the entry's spline radius is read only when some softening of this step
+  // reaches r (hmax: the largest radius of any particle or node)
+  if (r < hmax) {
+    const float he = *hep, h = he > hi ? he : hi;
+    if (r < h) fac = spline_fac_ir(r, ir, h);
+  }
+  float sfac;
+  if (C.poly) {
+    const float t = fmaf(r, C.tcoef, -1.0f);
+    float q = kSplitPoly[11];
+#pragma unroll
+    for (int i = 10; i >= 0; --i) q = fmaf(q, t, kSplitPoly[i]);
+    sfac = ex2_approx(r2 * C.nl2) * q;
+  } else {
+    sfac = split_factor(r * C.inv2rs, C.poly);
+  }
+  const float f = m * fac * sfac;
+  ax += f * dx;
+  ay += f * dy;
+  az += f * dz;
 }
 
 // Evaluate the list [0, len) for this lane's particle: the lane takes every
-// Sm-th entry from `sub`.  Entries are taken 32 at a time: a cheap pass tests
-// each against r_cut (and r > 0: the self pair) into a bit mask, then the lane
-// evaluates only the set bits, so the force arithmetic runs for in-range pairs
-// only and the warp iterates as often as its busiest lane has pairs in range.
-template <class R, bool kMasked>
-__device__ __forceinline__ void eval_list(const WalkSmem<R>& sm, int w, int len, int sub, int Sm, const Pos<R>& P,
-                                          R hi, R hmax, const WalkConst<R>& C, R& ax, R& ay, R& az,
-                                          unsigned& nin) {
+// Sm-th entry from `sub`.  Masked: entries are taken 32 at a time, a cheap pass
+// tests each against r_cut (and r > 0: the self pair) into a bit mask, then the
+// lane evaluates only the set bits, so the force arithmetic runs for in-range
+// pairs only and the warp iterates as often as its busiest lane has pairs in
+// range.
+template <bool kMasked>
+__device__ __forceinline__ void eval_list(const WalkSmem<float>& sm, int w, int len, int sub, int Sm,
+                                          const Pos<float>& P, float hi, float hmax, const WalkConst<float>& C,
+                                          float& ax, float& ay, float& az, unsigned& nin) {
   if (!kMasked) {
     // most entries in range (a group cube small against r_cut): one pass,
     // the force arithmetic guarded by the range test
     int e = sub;
     for (; e + Sm < len; e += 2 * Sm) {  // two entries per iteration (independent chains)
-      const LEntry<R> E0 = sm.e[w][e], E1 = sm.e[w][e + Sm];
-      R dx0, dy0, dz0, dx1, dy1, dz1;
-      const R r0 = entry_r2(E0, P, dx0, dy0, dz0);
-      const R r1 = entry_r2(E1, P, dx1, dy1, dz1);
+      const LEntry<float> E0 = sm.e[w][e], E1 = sm.e[w][e + Sm];
+      float dx0, dy0, dz0, dx1, dy1, dz1;
+      const float r0 = entry_r2(E0, P, dx0, dy0, dz0);
+      const float r1 = entry_r2(E1, P, dx1, dy1, dz1);
       if (in_range(r0, C.rcut2)) {
         ++nin;
         pair_force(dx0, dy0, dz0, r0, E0.m, &sm.h[w][e], hi, hmax, C, ax, ay, az);
@@ -333,9 +388,9 @@ __device__ __forceinline__ void eval_list(const WalkSmem<R>& sm, int w, int len,
       }
     }
     if (e < len) {
-      const LEntry<R> E0 = sm.e[w][e];
-      R dx, dy, dz;
-      const R r2 = entry_r2(E0, P, dx, dy, dz);
+      const LEntry<float> E0 = sm.e[w][e];
+      float dx, dy, dz;
+      const float r2 = entry_r2(E0, P, dx, dy, dz);
       if (in_range(r2, C.rcut2)) {
         ++nin;
         pair_force(dx, dy, dz, r2, E0.m, &sm.h[w][e], hi, hmax, C, ax, ay, az);
@@ -348,11 +403,11 @@ __device__ __forceinline__ void eval_list(const WalkSmem<R>& sm, int w, int len,
   for (int kb = 0; kb < nkmax; kb += 32) {
     unsigned mask = 0;
     const int kend = nk - kb < 32 ? nk - kb : 32;
-    const LEntry<R>* ep = &sm.e[w][sub + kb * Sm];
+    const LEntry<float>* ep = &sm.e[w][sub + kb * Sm];
 #pragma unroll 4
     for (int k = 0; k < kend; ++k) {
-      R dx, dy, dz;
-      const R r2 = entry_r2(ep[k * Sm], P, dx, dy, dz);
+      float dx, dy, dz;
+      const float r2 = entry_r2(ep[k * Sm], P, dx, dy, dz);
       mask |= in_range(r2, C.rcut2) ? (1u << k) : 0u;
     }
     nin += __popc(mask);
@@ -361,7 +416,36 @@ __device__ __forceinline__ void eval_list(const WalkSmem<R>& sm, int w, int len,
         const int k = __ffs(mask) - 1;
         mask &= mask - 1u;
         const int e = sub + (kb + k) * Sm;
-        pair_in_range(sm.e[w][e], &sm.h[w][e], P, hi, hmax, C, ax, ay, az);
+        const LEntry<float> E = sm.e[w][e];
+        float dx, dy, dz;
+        const float r2 = entry_r2(E, P, dx, dy, dz);
+        pair_force(dx, dy, dz, r2, E.m, &sm.h[w][e], hi, hmax, C, ax, ay, az);
+      }
+    }
+  }
+}
+
+// FP64 (one form for every walk_eval): 64 entries at a time, nearly the whole
+// list of a lane; the FP32 bound fills the mask.  The warp iterates as often
+// as its busiest lane, so one long mask beats two short ones.
+template <bool kMasked>
+__device__ __forceinline__ void eval_list(const WalkSmem<double>& sm, int w, int len, int sub, int Sm,
+                                          const Pos<double>& P, double hi, double hmax, const WalkConst<double>& C,
+                                          double& ax, double& ay, double& az, unsigned& nin) {
+  const int nk = sub < len ? (len - sub + Sm - 1) / Sm : 0;
+  const int nkmax = __reduce_max_sync(0xffffffffu, (unsigned)nk);
+  for (int kb = 0; kb < nkmax; kb += 64) {
+    unsigned long long mask = 0;
+    const int kend = nk - kb < 64 ? nk - kb : 64;
+    const LEntry<double>* ep = &sm.e[w][sub + kb * Sm];
+#pragma unroll 4
+    for (int k = 0; k < kend; ++k) mask |= maybe_in_range(ep[k * Sm], P, C.rcut2_hi) ? (1ull << k) : 0ull;
+    while (__any_sync(0xffffffffu, mask != 0ull)) {
+      if (mask) {
+        const int k = __ffsll((long long)mask) - 1;
+        mask &= mask - 1ull;
+        const int e = sub + (kb + k) * Sm;
+        pair_fp64(sm.e[w][e], &sm.h[w][e], P, hi, hmax, C, ax, ay, az, nin);
       }
     }
   }
@@ -639,7 +723,7 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 8 : 5) k_walk(
 #define DZS_WALK_FLUSH()                                                     \
   do {                                                                       \
     __syncwarp();                                                            \
-    eval_list<R, kMasked>(sm, w, len, sub, Sm, P, hi, hmax, C, ax, ay, az, nin); \
+    eval_list<kMasked>(sm, w, len, sub, Sm, P, hi, hmax, C, ax, ay, az, nin);    \
     if (lane == 0) npairs += (unsigned)len * (unsigned)cnt;                  \
     glen += len;                                                             \
     len = 0;                                                                 \
@@ -873,6 +957,15 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
   C.tcoef = (R)(s / (2.0 * c->rs) * (2.0 / (double)kSplitXMax));
   C.nl2 = (R)(-1.4426950408889634 * (s / (2.0 * c->rs)) * (s / (2.0 * c->rs)));
   C.gm0 = (R)(c->gm0 / (s * s));
+  C.zscale = C.igscale = (R)1;
+  C.rcut2_hi = 0.f;
+  if (sizeof(R) == 8) {
+    const double x1 = s / (2.0 * c->rs);
+    C.zscale = (R)(x1 * x1);
+    C.igscale = (R)(1.0 / (x1 * x1 * x1));
+    C.gm0 = (R)((double)C.gm0 * (x1 * x1 * x1));
+    C.rcut2_hi = std::nextafter((float)((double)C.rcut2 * (1.0 + 0x1p-20)), INFINITY);
+  }
   C.kick = close_kick ? (R)c->T.kick2[step] : (R)0;
   C.skip_d2 = c->walk_skip_d2;
   for (int l = 0; l <= kMaxLevel; ++l) C.open_d2[l] = c->walk_open_d2[l];
@@ -971,11 +1064,13 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
   // particle set (leaves of ~B particles, side ~2 spacings) are at least
   // r_cut / 2 wide; both evaluate the same pairs in the same order
   const double spacing = c->P.box / c->P.n1d;
-  const bool masked = c->P.walk_eval == DZS_WALK_MASKED ||
-                      (c->P.walk_eval == DZS_WALK_AUTO && 4.0 * spacing >= c->rcut);
+  const bool masked = c->fp64 || c->P.walk_eval == DZS_WALK_MASKED ||
+                      (c->P.walk_eval == DZS_WALK_AUTO && 4.0 * spacing >= c->rcut);  // FP64 has one form
   const bool diag = c->walk_diag;
-  auto kern = masked ? (diag ? k_walk<R, true, true> : k_walk<R, true, false>)
-                     : (diag ? k_walk<R, false, true> : k_walk<R, false, false>);
+  auto kern = diag ? k_walk<R, true, true> : k_walk<R, true, false>;
+  if constexpr (sizeof(R) == 4) {
+    if (!masked) kern = diag ? k_walk<R, false, true> : k_walk<R, false, false>;
+  }
   size_t sm = sizeof(WalkSmem<R>);
   static bool attr_done[2][2][2] = {};
   if (!attr_done[sizeof(R) == 8][masked][diag]) {
@@ -994,7 +1089,55 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
                                                   (unsigned long long*)(c->B.counters + 4), c->B.wlen);
 }
 
+// coefficients of F on each cell of z: Chebyshev interpolation in the cell's
+// own variable, rewritten in powers of z - (cell middle)
+void fill_ztab(double (*tab)[kZDeg + 1]) {
+  typedef long double ld;
+  constexpr int n = kZDeg + 1;
+  const ld pi = 3.14159265358979323846264338327950288L, tsp = 1.12837916709551257389615890312154517L;
+  ld node[n], cheb[n][n];  // cheb[j][p]: coefficient of tau^p in T_j
+  for (int k = 0; k < n; ++k) node[k] = cosl(pi * (k + 0.5L) / n);
+  for (int j = 0; j < n; ++j)
+    for (int p = 0; p < n; ++p)
+      cheb[j][p] = j == 0 ? (p == 0 ? 1.0L : 0.0L)
+                 : j == 1 ? (p == 1 ? 1.0L : 0.0L)
+                          : (p > 0 ? 2.0L * cheb[j - 1][p - 1] : 0.0L) - cheb[j - 2][p];
+  for (int c = 0; c < kZCells; ++c) {
+    const ld width = ldexpl(1.0L / kZSub, kZLo + c / kZSub), half = 0.5L * width;
+    const ld mid = ldexpl(1.0L, kZLo + c / kZSub) + width * (c % kZSub) + half;
+    ld f[n], mono[n] = {0};
+    for (int k = 0; k < n; ++k) {
+      const ld z = mid + half * node[k], x = sqrtl(z);
+      f[k] = (erfcl(x) + tsp * x * expl(-z)) / (z * x);
+    }
+    for (int j = 0; j < n; ++j) {
+      ld a = 0.0L;
+      for (int k = 0; k < n; ++k) a += f[k] * cosl(pi * j * (k + 0.5L) / n);
+      a *= (j == 0 ? 1.0L : 2.0L) / n;
+      for (int p = 0; p <= j; ++p) mono[p] += a * cheb[j][p];
+    }
+    ld scale = 1.0L;
+    for (int p = 0; p < n; ++p, scale /= half) tab[c][p] = (double)(mono[p] * scale);
+  }
+}
+
 }  // namespace
+
+// the FP64 pair table, once per device (any thread may create a context)
+bool upload_walk_constants(int dev) {
+  static std::mutex mu;
+  static bool done[256] = {false};
+  static std::vector<double> host;
+  std::lock_guard<std::mutex> lock(mu);
+  if (dev < 0 || dev >= 256) return false;
+  if (done[dev]) return true;
+  if (host.empty()) {
+    host.resize((size_t)kZCells * (kZDeg + 1));
+    fill_ztab(reinterpret_cast<double(*)[kZDeg + 1]>(host.data()));
+  }
+  done[dev] = cudaMemcpyToSymbol(kZTab, host.data(), host.size() * sizeof(double)) == cudaSuccess;
+  return done[dev];
+}
 
 void launch_walk(dzs_ctx* c, bool tree, bool close_kick, int step) {
   c->launches += 2;
