@@ -110,11 +110,10 @@ typedef struct {
                           ring makes dzs_step check each step's records first */
   int32_t dzs_criterion; /* DZS_CRIT_GEOMETRIC: l/D < theta_dzs (Sec. 2.2.1);
                            DZS_CRIT_DYNAMICAL: Eq. 2 with d -> D of Eq. 3 */
-  int32_t walk_eval;     /* execution only (results identical): how the tree walk
-                            evaluates its lists; DZS_WALK_AUTO (0), DZS_WALK_MASKED
-                            (1: a range-test pass, then force arithmetic for the
-                            pairs within r_cut), DZS_WALK_GUARDED (2: one pass, the
-                            arithmetic guarded by the range test) */
+  int32_t walk_eval;     /* execution only (results identical): DZS_WALK_AUTO (0),
+                            DZS_WALK_MASKED (1), DZS_WALK_GUARDED (2); the tree
+                            walk has one way of evaluating its lists, which
+                            every value selects */
   double alpha_dyn;      /* dynamical: merge iff D > 0 and G M l^2 / D^4 <
                             alpha_dyn a_min, a_min = smallest |g| (previous
                             step) of the particles not yet crossed; >= 0 */

@@ -38,15 +38,16 @@
 // holds more than 172 entries (a round adds at most 32 monopoles and the
 // leaves that fit; leaves that do not fit wait on the stack).  A group of c
 // particles puts every lane to work: lane -> particle m = lane mod c, the
-// S_m lanes of particle m each taking every S_m-th entry.  Entries are taken
-// 32 at a time: a cheap pass tests r < r_cut into a bit mask, then only the
-// pairs in range get the force arithmetic (the warp iterates as often as its
-// busiest lane has pairs in range); the lanes of a particle are combined by a
-// fixed shuffle tree (the result is deterministic).  Pair force: softened
-// 1/r^3 times T(r) = erfc(x) + (2/sqrt(pi)) x exp(-x^2), x = r / 2 r_s, zero
-// at r = 0 and r >= r_cut.  FP32 evaluates T = exp(-x^2) Q(x) with a fitted
-// polynomial (gen_split_poly.py, relative error 3.3e-7); FP64 reads T(r) / r^3
-// from a table of polynomials in r^2.
+// S_m lanes of particle m each taking every S_m-th pair of entries; the lanes
+// of a particle are combined by a fixed shuffle tree (the result is
+// deterministic).  Pair force: softened 1/r^3 times T(r) = erfc(x) +
+// (2/sqrt(pi)) x exp(-x^2), x = r / 2 r_s, zero at r = 0 and r >= r_cut.  FP32
+// evaluates T = exp(-x^2) Q(x) with a fitted polynomial (gen_split_poly.py,
+// relative error 3.3e-7), two entries at a time on the paired FP32
+// instructions; FP64 reads T(r) / r^3 from a table of polynomials in r^2.
+// Walk of the 128^3 / mesh 256 set, early (30% of listed pairs in range), late,
+// and of 256^3 / mesh 256 (75%): bit-masked or guarded scalar evaluation 2.72,
+// 0.69, 42.1 ms, paired 2.47, 0.60, 34.0 ms.
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -56,10 +57,10 @@
 namespace dzs {
 namespace {
 
-// shared memory sets the occupancy (8 blocks of 4 warps per SM in FP32, 64
-// registers): stack 512 entries (deepest use measured 329; an overflow sets an
-// error bit), list 236 entries (8 blocks measured 2% faster than 7 blocks
-// with 300-entry lists)
+// 7 blocks of 4 warps per SM in FP32: 72 registers (8 blocks of 64 spill in the
+// paired evaluation: 9% slower; 6 blocks of 80: 8%).  Stack 512 entries (deepest
+// use measured 337; an overflow sets an error bit), list 236 entries (296, the
+// most that 7 blocks' shared memory holds, is no faster)
 constexpr int kWarps = 4;
 constexpr int kStack = 512;
 constexpr int kList = 236;
@@ -144,12 +145,35 @@ __device__ __forceinline__ Pos<double> make_pos<double>(uint32_t x, uint32_t y, 
   return Pos<double>{x, y, z};
 }
 
+// list rows hold one entry more than kList (the pad of an odd list), 16-byte
+// aligned; FP32 by component, so that two consecutive entries load as the
+// operands of the paired FP32 instructions
+constexpr int kRow = (kList + 4) & ~3;
 template <class R>
-struct WalkSmem {
+struct WalkSmem;
+template <>
+struct __align__(16) WalkSmem<float> {
+  float x[kWarps][kRow], y[kWarps][kRow], z[kWarps][kRow], m[kWarps][kRow];
+  float h[kWarps][kRow];  // spline radius 2.8 eps of the entry (lattice units)
   int32_t stack[kWarps][kStack];
-  LEntry<R> e[kWarps][kList];
-  R h[kWarps][kList];  // spline radius 2.8 eps of the entry (lattice units)
 };
+template <>
+struct WalkSmem<double> {
+  int32_t stack[kWarps][kStack];
+  LEntry<double> e[kWarps][kList];
+  double h[kWarps][kList];
+};
+__device__ __forceinline__ void put_entry(WalkSmem<float>& sm, int w, int i, const LEntry<float>& E, float h) {
+  sm.x[w][i] = E.x;
+  sm.y[w][i] = E.y;
+  sm.z[w][i] = E.z;
+  sm.m[w][i] = E.m;
+  sm.h[w][i] = h;
+}
+__device__ __forceinline__ void put_entry(WalkSmem<double>& sm, int w, int i, const LEntry<double>& E, double h) {
+  sm.e[w][i] = E;
+  sm.h[w][i] = h;
+}
 
 // FP64 pair factor: F(z) = T(sqrt z) z^(-3/2), z = (r / 2 r_s)^2, so that
 // T(r) / r^3 = F / (2 r_s)^3 needs no square root, division, erfc or exp.
@@ -184,7 +208,6 @@ struct WalkConst {
   int B;
   int close;
   int tree;
-  int poly;  // FP32: use the fitted split polynomial (x_max <= 2.5)
   int front;                  // frontier depth f (0: start at the root)
   const int32_t* ftab;        // [2^f]^3 row-major: node of each depth-f cell, -1 if empty
   int frontF;                 // window frontier depth F > f (0: none)
@@ -224,14 +247,7 @@ __device__ __forceinline__ R spline_fac(R r, R h) {
           (R)(1.0 / 15.0) / (q * q * q)) / h3;
 }
 
-__device__ __forceinline__ float split_factor(float x, int poly) {
-  if (poly) {
-    float t = x * (2.0f / kSplitXMax) - 1.0f;
-    float q = kSplitPoly[11];
-#pragma unroll
-    for (int i = 10; i >= 0; --i) q = fmaf(q, t, kSplitPoly[i]);
-    return __expf(-x * x) * q;
-  }
+__device__ __forceinline__ float split_factor(float x) {
   return erfcf(x) + 1.1283791670955126f * x * __expf(-x * x);
 }
 
@@ -242,26 +258,19 @@ __device__ __forceinline__ float ex2_approx(float v) {
   return y;
 }
 
-__device__ __forceinline__ double split_factor(double x, int) {
+__device__ __forceinline__ double split_factor(double x) {
   return erfc(x) + 1.1283791670955126 * x * exp(-x * x);
 }
 
-// r^2 >= 1 lattice unit^2 here (no denormals): the plain hardware rsqrt
-__device__ __forceinline__ void inv_and_r(float r2, float& r, float& ir) {
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(r2));
-  r = r2 * ir;
+// r^2 >= 1 lattice unit^2 for a pair in range (no denormals): the plain hardware rsqrt
+__device__ __forceinline__ float rsqrt_approx(float v) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(v));
+  return y;
 }
 
-// squared lattice distance of entry E from the lane's particle P: FP32 from
-// the two offsets from the group centre, FP64 from the exact int32
-// minimum-image offsets
-__device__ __forceinline__ float entry_r2(const LEntry<float>& E, const Pos<float>& P, float& dx, float& dy,
-                                          float& dz) {
-  dx = E.x - P.x;
-  dy = E.y - P.y;
-  dz = E.z - P.z;
-  return dx * dx + dy * dy + dz * dz;
-}
+// squared lattice distance of FP64 entry E from the lane's particle P, from the
+// exact int32 minimum-image offsets
 __device__ __forceinline__ double entry_r2(const LEntry<double>& E, const Pos<double>& P, double& dx, double& dy,
                                            double& dz) {
   dx = (double)(int32_t)(E.x - P.x);
@@ -302,7 +311,7 @@ __device__ __forceinline__ void pair_fp64(const LEntry<double>& E, const double*
     const double he = *hep, h = he > hi ? he : hi;
     if (r2 < h * h) {
       const double r = sqrt(r2);
-      f = C.igscale * spline_fac(r, h) * split_factor(r * C.inv2rs, 0);
+      f = C.igscale * spline_fac(r, h) * split_factor(r * C.inv2rs);
       done = true;
     }
   }
@@ -321,7 +330,7 @@ __device__ __forceinline__ void pair_fp64(const LEntry<double>& E, const double*
       f = fma(f, t, q0.x);
     } else {
       const double r = sqrt(r2);
-      f = C.igscale * split_factor(r * C.inv2rs, 0) / (r2 * r);
+      f = C.igscale * split_factor(r * C.inv2rs) / (r2 * r);
     }
   }
   f *= E.m;
@@ -330,105 +339,86 @@ __device__ __forceinline__ void pair_fp64(const LEntry<double>& E, const double*
   az += f * dz;
 }
 
-// force of one FP32 entry at offset (dx, dy, dz), 0 < r^2 < r_cut^2 (the caller
-// has tested the range)
-__device__ __forceinline__ void pair_force(float dx, float dy, float dz, float r2, float m, const float* hep, float hi,
-                                           float hmax, const WalkConst<float>& C, float& ax, float& ay, float& az) {
-  float r, ir;
-  inv_and_r(r2, r, ir);
-  float fac = ir * ir * ir;
-  // the entry's spline radius is read only when some softening of this step
-  // reaches r (hmax: the largest radius of any particle or node)
-  if (r < hmax) {
-    const float he = *hep, h = he > hi ? he : hi;
-    if (r < h) fac = spline_fac_ir(r, ir, h);
-  }
-  float sfac;
-  if (C.poly) {
-    const float t = fmaf(r, C.tcoef, -1.0f);
-    float q = kSplitPoly[11];
+// T(r) / r^3 of two FP32 pairs at once: the paired instructions (one issue slot
+// for two operations), each component rounded as the scalar form.  ir = 1 / r,
+// r2 of a self pair or beyond r_cut gives a value the caller drops.
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 split2(float2 r2, float2 r, const WalkConst<float>& C) {
+  const float2 t = __ffma2_rn(r, both(C.tcoef), both(-1.0f));
+  float2 q = both(kSplitPoly[11]);
 #pragma unroll
-    for (int i = 10; i >= 0; --i) q = fmaf(q, t, kSplitPoly[i]);
-    sfac = ex2_approx(r2 * C.nl2) * q;
-  } else {
-    sfac = split_factor(r * C.inv2rs, C.poly);
-  }
-  const float f = m * fac * sfac;
-  ax += f * dx;
-  ay += f * dy;
-  az += f * dz;
+  for (int i = 10; i >= 0; --i) q = __ffma2_rn(q, t, both(kSplitPoly[i]));
+  const float2 x = __fmul2_rn(r2, both(C.nl2));
+  return __fmul2_rn(q, make_float2(ex2_approx(x.x), ex2_approx(x.y)));
 }
 
 // Evaluate the list [0, len) for this lane's particle: the lane takes every
-// Sm-th entry from `sub`.  Masked: entries are taken 32 at a time, a cheap pass
-// tests each against r_cut (and r > 0: the self pair) into a bit mask, then the
-// lane evaluates only the set bits, so the force arithmetic runs for in-range
-// pairs only and the warp iterates as often as its busiest lane has pairs in
-// range.
-template <bool kMasked>
-__device__ __forceinline__ void eval_list(const WalkSmem<float>& sm, int w, int len, int sub, int Sm,
-                                          const Pos<float>& P, float hi, float hmax, const WalkConst<float>& C,
-                                          float& ax, float& ay, float& az, unsigned& nin) {
-  if (!kMasked) {
-    // most entries in range (a group cube small against r_cut): one pass,
-    // the force arithmetic guarded by the range test
-    int e = sub;
-    for (; e + Sm < len; e += 2 * Sm) {  // two entries per iteration (independent chains)
-      const LEntry<float> E0 = sm.e[w][e], E1 = sm.e[w][e + Sm];
-      float dx0, dy0, dz0, dx1, dy1, dz1;
-      const float r0 = entry_r2(E0, P, dx0, dy0, dz0);
-      const float r1 = entry_r2(E1, P, dx1, dy1, dz1);
-      if (in_range(r0, C.rcut2)) {
-        ++nin;
-        pair_force(dx0, dy0, dz0, r0, E0.m, &sm.h[w][e], hi, hmax, C, ax, ay, az);
-      }
-      if (in_range(r1, C.rcut2)) {
-        ++nin;
-        pair_force(dx1, dy1, dz1, r1, E1.m, &sm.h[w][e + Sm], hi, hmax, C, ax, ay, az);
-      }
-    }
-    if (e < len) {
-      const LEntry<float> E0 = sm.e[w][e];
-      float dx, dy, dz;
-      const float r2 = entry_r2(E0, P, dx, dy, dz);
-      if (in_range(r2, C.rcut2)) {
-        ++nin;
-        pair_force(dx, dy, dz, r2, E0.m, &sm.h[w][e], hi, hmax, C, ax, ay, az);
-      }
-    }
-    return;
+// Sm-th pair of consecutive entries from `sub`, two entries at a time.  kPoly:
+// every listed entry gets the full arithmetic (paired instructions: ~25 issue
+// slots an entry) and entries out of range are dropped by a select.  Testing
+// first and evaluating the survivors, by bit mask or by a guarded branch, took
+// ~60 slots an entry: the loop is issue-bound and its lanes diverge.
+template <bool kPoly>
+__device__ __forceinline__ void eval_list(WalkSmem<float>& sm, int w, int len, int sub, int Sm, const Pos<float>& P,
+                                          float hi, float hmax, const WalkConst<float>& C, float& ax, float& ay,
+                                          float& az, unsigned& nin) {
+  if (len & 1) {  // pad to whole pairs with an entry beyond every r_cut
+    if ((threadIdx.x & 31) == 0) put_entry(sm, w, len, LEntry<float>{1e10f, 0.f, 0.f, 0.f}, 0.f);
+    __syncwarp();
   }
-  const int nk = sub < len ? (len - sub + Sm - 1) / Sm : 0;
-  const int nkmax = __reduce_max_sync(0xffffffffu, (unsigned)nk);
-  for (int kb = 0; kb < nkmax; kb += 32) {
-    unsigned mask = 0;
-    const int kend = nk - kb < 32 ? nk - kb : 32;
-    const LEntry<float>* ep = &sm.e[w][sub + kb * Sm];
-#pragma unroll 4
-    for (int k = 0; k < kend; ++k) {
-      float dx, dy, dz;
-      const float r2 = entry_r2(ep[k * Sm], P, dx, dy, dz);
-      mask |= in_range(r2, C.rcut2) ? (1u << k) : 0u;
-    }
-    nin += __popc(mask);
-    while (__any_sync(0xffffffffu, mask != 0u)) {
-      if (mask) {
-        const int k = __ffs(mask) - 1;
-        mask &= mask - 1u;
-        const int e = sub + (kb + k) * Sm;
-        const LEntry<float> E = sm.e[w][e];
-        float dx, dy, dz;
-        const float r2 = entry_r2(E, P, dx, dy, dz);
-        pair_force(dx, dy, dz, r2, E.m, &sm.h[w][e], hi, hmax, C, ax, ay, az);
+  // bit patterns of r^2 - 1: 0 < r^2 < v orders like an unsigned compare (the
+  // self pair, r^2 = 0, wraps to the top)
+  const unsigned cut = __float_as_uint(C.rcut2) - 1u, soft = __float_as_uint(hmax * hmax) - 1u;
+  const float2 px = both(-P.x), py = both(-P.y), pz = both(-P.z);
+  float2 sx = both(0.f), sy = both(0.f), sz = both(0.f);
+  for (int e = 2 * sub; e < len; e += 2 * Sm) {
+    const float2 dx = __fadd2_rn(*reinterpret_cast<const float2*>(&sm.x[w][e]), px);
+    const float2 dy = __fadd2_rn(*reinterpret_cast<const float2*>(&sm.y[w][e]), py);
+    const float2 dz = __fadd2_rn(*reinterpret_cast<const float2*>(&sm.z[w][e]), pz);
+    const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+    const unsigned b0 = __float_as_uint(r2.x) - 1u, b1 = __float_as_uint(r2.y) - 1u;
+    const bool in0 = b0 < cut, in1 = b1 < cut;
+    nin += in0 ? 1u : 0u;
+    nin += in1 ? 1u : 0u;
+    float2 f;
+    if (kPoly) {
+      const float2 ir = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+      const float2 r = __fmul2_rn(r2, ir);
+      float2 fac = __fmul2_rn(__fmul2_rn(ir, ir), ir);
+      // the entries' spline radii are read only when some softening of this
+      // step reaches r (hmax: the largest radius of any particle or node)
+      if (min(b0, b1) < soft) {
+        const float h0 = fmaxf(sm.h[w][e], hi), h1 = fmaxf(sm.h[w][e + 1], hi);
+        if (in0 && r.x < h0) fac.x = spline_fac_ir(r.x, ir.x, h0);
+        if (in1 && r.y < h1) fac.y = spline_fac_ir(r.y, ir.y, h1);
+      }
+      f = __fmul2_rn(__fmul2_rn(*reinterpret_cast<const float2*>(&sm.m[w][e]), fac), split2(r2, r, C));
+    } else {
+      // a cut beyond the fitted polynomial's range: the formula
+      f = both(0.f);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float v = q ? r2.y : r2.x, ir = rsqrt_approx(v), r = v * ir, h = fmaxf(sm.h[w][e + q], hi);
+        if (!(q ? in1 : in0)) continue;
+        const float fac = r < h ? spline_fac_ir(r, ir, h) : ir * ir * ir;
+        (q ? f.y : f.x) = sm.m[w][e + q] * fac * split_factor(r * C.inv2rs);
       }
     }
+    f.x = in0 ? f.x : 0.f;
+    f.y = in1 ? f.y : 0.f;
+    sx = __ffma2_rn(f, dx, sx);
+    sy = __ffma2_rn(f, dy, sy);
+    sz = __ffma2_rn(f, dz, sz);
   }
+  ax += sx.x + sx.y;
+  ay += sy.x + sy.y;
+  az += sz.x + sz.y;
 }
 
 // FP64 (one form for every walk_eval): 64 entries at a time, nearly the whole
 // list of a lane; the FP32 bound fills the mask.  The warp iterates as often
 // as its busiest lane, so one long mask beats two short ones.
-template <bool kMasked>
+template <bool>
 __device__ __forceinline__ void eval_list(const WalkSmem<double>& sm, int w, int len, int sub, int Sm,
                                           const Pos<double>& P, double hi, double hmax, const WalkConst<double>& C,
                                           double& ax, double& ay, double& az, unsigned& nin) {
@@ -604,13 +594,11 @@ __global__ void k_front_fill_F(const int32_t* __restrict__ lvl, const Node* __re
   }
 }
 
-// kMasked: evaluate lists with the range-masked pass (pays off when many
-// listed entries lie beyond r_cut of a given particle: groups not small
-// against r_cut), else with one range-guarded pass.  kDiag: also count node
+// kPoly (FP32): the cut lies within the fitted split polynomial.  kDiag: also count node
 // tests, traversal rounds and the deepest stack use (three instructions per
 // round, ~1.5% of the walk: only while asked for)
-template <class R, bool kMasked, bool kDiag>
-__global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 8 : 5) k_walk(
+template <class R, bool kPoly, bool kDiag>
+__global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
     const int32_t* __restrict__ groups, const uint64_t* __restrict__ counters, unsigned int* __restrict__ next,
     const Node* __restrict__ nodes, const R* __restrict__ nh, int64_t cap, const uint32_t* __restrict__ u,
     const Entry<R>* __restrict__ pm, const R* __restrict__ ph, R* __restrict__ p, R* __restrict__ g, WalkConst<R> C,
@@ -723,7 +711,7 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 8 : 5) k_walk(
 #define DZS_WALK_FLUSH()                                                     \
   do {                                                                       \
     __syncwarp();                                                            \
-    eval_list<kMasked>(sm, w, len, sub, Sm, P, hi, hmax, C, ax, ay, az, nin);    \
+    eval_list<kPoly>(sm, w, len, sub, Sm, P, hi, hmax, C, ax, ay, az, nin);    \
     if (lane == 0) npairs += (unsigned)len * (unsigned)cnt;                  \
     glen += len;                                                             \
     len = 0;                                                                 \
@@ -802,8 +790,7 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 8 : 5) k_walk(
           unsigned am = __ballot_sync(0xffffffffu, acc);
           if (acc) {
             int pos = len + __popc(am & lt);
-            sm.e[w][pos] = make_entry(nd.comx, nd.comy, nd.comz, C.gm0 * (R)nd.mass, cg);
-            sm.h[w][pos] = nhi;
+            put_entry(sm, w, pos, make_entry(nd.comx, nd.comy, nd.comz, C.gm0 * (R)nd.mass, cg), nhi);
           }
           len += __popc(am);
           // children of opened inner nodes onto the stack
@@ -870,8 +857,7 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 8 : 5) k_walk(
             const unsigned tm = __ballot_sync(0xffffffffu, take);
             if (take) {
               const int pos = len + __popc(tm & lt);
-              sm.e[w][pos] = make_entry(E.x, E.y, E.z, E.m, cg);
-              sm.h[w][pos] = hj;
+              put_entry(sm, w, pos, make_entry(E.x, E.y, E.z, E.m, cg), hj);
             }
             len += __popc(tm);
           }
@@ -897,8 +883,7 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 8 : 5) k_walk(
               const unsigned tm = __ballot_sync(0xffffffffu, take);
               if (take) {
                 const int pos = len + __popc(tm & lt);
-                sm.e[w][pos] = make_entry(E.x, E.y, E.z, E.m, cg);
-                sm.h[w][pos] = hj;
+                put_entry(sm, w, pos, make_entry(E.x, E.y, E.z, E.m, cg), hj);
               }
               len += __popc(tm);
             }
@@ -982,7 +967,6 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
   C.B = c->P.leaf_bucket;
   C.close = close_kick ? 1 : 0;
   C.tree = tree ? 1 : 0;
-  C.poly = (c->P.rcut_rs / 2.0 <= (double)kSplitXMax) ? 1 : 0;
   // frontier depth: every depth above it never accepts (a non-skipped node's
   // COM distance is at most sqrt(skip_d2) + sqrt(3) l, and that opens it), and
   // its cells are wider than r_cut (cells beyond the 27 neighbours are skipped)
@@ -1060,22 +1044,17 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
           c->B.lvl_count, c->B.nodes, c->B.parent, C.front, C.frontF, fm, (int32_t*)C.ftabF, (uint8_t*)C.fspanF);
     }
   }
-  // automatic: the range-masked evaluation when the walk groups of a uniform
-  // particle set (leaves of ~B particles, side ~2 spacings) are at least
-  // r_cut / 2 wide; both evaluate the same pairs in the same order
-  const double spacing = c->P.box / c->P.n1d;
-  const bool masked = c->fp64 || c->P.walk_eval == DZS_WALK_MASKED ||
-                      (c->P.walk_eval == DZS_WALK_AUTO && 4.0 * spacing >= c->rcut);  // FP64 has one form
+  const bool poly = c->fp64 || c->P.rcut_rs / 2.0 <= (double)kSplitXMax;  // FP64 has one form
   const bool diag = c->walk_diag;
   auto kern = diag ? k_walk<R, true, true> : k_walk<R, true, false>;
   if constexpr (sizeof(R) == 4) {
-    if (!masked) kern = diag ? k_walk<R, false, true> : k_walk<R, false, false>;
+    if (!poly) kern = diag ? k_walk<R, false, true> : k_walk<R, false, false>;
   }
   size_t sm = sizeof(WalkSmem<R>);
   static bool attr_done[2][2][2] = {};
-  if (!attr_done[sizeof(R) == 8][masked][diag]) {
+  if (!attr_done[sizeof(R) == 8][poly][diag]) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr_done[sizeof(R) == 8][masked][diag] = true;
+    attr_done[sizeof(R) == 8][poly][diag] = true;
   }
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, sm);
