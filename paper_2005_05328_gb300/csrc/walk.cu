@@ -461,13 +461,15 @@ __device__ __forceinline__ bool near_group(uint32_t px, uint32_t py, uint32_t pz
   return exact_d2(dv) <= C.skip_d2;
 }
 
-template <class R>
-__device__ __forceinline__ int warp_incl_scan(int v, int lane) {
+// the shuffle's own predicate (source lane exists) guards the addition
+__device__ __forceinline__ int warp_incl_scan(int v) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int t = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v += t;
-  }
+  for (int o = 1; o < 32; o <<= 1)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
+        "shfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t@p add.s32 %0, %0, t;\n\t}"
+        : "+r"(v)
+        : "r"(o));
   return v;
 }
 
@@ -600,8 +602,8 @@ __global__ void k_front_fill_F(const int32_t* __restrict__ lvl, const Node* __re
 template <class R, bool kPoly, bool kDiag>
 __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
     const int32_t* __restrict__ groups, const uint64_t* __restrict__ counters, unsigned int* __restrict__ next,
-    const Node* __restrict__ nodes, const R* __restrict__ nh, int64_t cap, const uint32_t* __restrict__ u,
-    const Entry<R>* __restrict__ pm, const R* __restrict__ ph, R* __restrict__ p, R* __restrict__ g, WalkConst<R> C,
+    const Node* __restrict__ nodes, const R* __restrict__ nh, int64_t cap, const Entry<R>* __restrict__ pm,
+    const R* __restrict__ ph, R* __restrict__ p, R* __restrict__ g, WalkConst<R> C,
     uint32_t* __restrict__ err, unsigned long long* __restrict__ pairs, int32_t* __restrict__ wlen) {
   extern __shared__ unsigned char smem_raw[];
   WalkSmem<R>& sm = *reinterpret_cast<WalkSmem<R>*>(smem_raw);
@@ -631,7 +633,8 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
       const int m = lane % cnt, sub = lane / cnt;
       const int Sm = 32 / cnt + (m < 32 % cnt ? 1 : 0);
       const int i = gn.start + c0 + m;
-      const Pos<R> P = make_pos<R>(u[i], u[cap + i], u[2 * cap + i], cg);
+      const Entry<R> pi = pm[i];  // one vector load for the position
+      const Pos<R> P = make_pos<R>(pi.x, pi.y, pi.z, cg);
       const R hi = ph[i];
       R ax = 0, ay = 0, az = 0;
       if (C.tree) {
@@ -654,14 +657,16 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
           }
           if (na[0] <= 6u && na[1] <= 6u && na[2] <= 6u) {
             const int nyz = (int)(na[1] * na[2]), total = (int)na[0] * nyz;
+            const float inyz = 1.0f / (float)nyz, inz = 1.0f / (float)na[2];
             bool bad = false;
             for (int b = 0; b < total; b += 32) {
               const int q = b + lane;
               bool push = false;
               int ni = -1;
               if (q < total) {
-                const uint32_t qx = (uint32_t)(q / nyz), qr = (uint32_t)(q - (int)qx * nyz);
-                const uint32_t qy = qr / na[2], qz = qr - qy * na[2];
+                // exact for q < 216: the quotient is at least 1/36 from an integer above
+                const uint32_t qx = (uint32_t)(((float)q + 0.5f) * inyz), qr = (uint32_t)(q - (int)qx * nyz);
+                const uint32_t qy = (uint32_t)(((float)qr + 0.5f) * inz), qz = qr - qy * na[2];
                 const uint32_t x = (lo[0] + qx) & Dm, y = (lo[1] + qy) & Dm, z = (lo[2] + qz) & Dm;
                 const int64_t cell = ((int64_t)x * (Dm + 1) + y) * (Dm + 1) + z;
                 ni = C.ftabF[cell];
@@ -798,7 +803,7 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
           // the low half, leaf particles (<= B <= 14 per lane) in the high half
           int nch = inner ? (int)((nd.meta >> 8) & 0xff) : 0;
           int lc = (leaf && nd.count <= C.B) ? nd.count : 0;
-          const int both = warp_incl_scan<R>(nch | (lc << 16), lane);
+          const int both = warp_incl_scan(nch | (lc << 16));
           int ex = (both & 0xffff) - nch;
           int tot = __shfl_sync(0xffffffffu, both & 0xffff, 31);
           const int incl = both >> 16;
@@ -1063,8 +1068,7 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
   int grid = (per_sm > 0 ? per_sm : 1) * (nsm > 0 ? nsm : 1);
   unsigned int* next = (unsigned int*)(c->B.counters + 6);
   cudaMemsetAsync(next, 0, sizeof(unsigned int), c->stream);
-  kern<<<grid, kWarps * 32, sm, c->stream>>>(c->B.groups, c->B.counters, next, c->B.nodes, nh, c->cap, c->B.u,
-                                                  pm, ph, (R*)c->B.p, (R*)c->B.g, C, c->B.err,
+  kern<<<grid, kWarps * 32, sm, c->stream>>>(c->B.groups, c->B.counters, next, c->B.nodes, nh, c->cap, pm, ph, (R*)c->B.p, (R*)c->B.g, C, c->B.err,
                                                   (unsigned long long*)(c->B.counters + 4), c->B.wlen);
 }
 
