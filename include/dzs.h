@@ -487,8 +487,8 @@ DZS_API dzs_status dzs_set_profiling(dzs_ctx* c, int32_t enable);
 DZS_API dzs_status dzs_get_profile(dzs_ctx* c, double ms[DZS_PROF_N], uint64_t calls[DZS_PROF_N]);
 
 /* Largest n accepted by dzs_morton_sort_noalloc.  Its scratch is a static
- * device array of 24 * n + 4 * (257 * ceil(n / 2048) + 256) + 256 bytes,
- * about 6.4 MB, which every GPU that loads the library holds until exit. */
+ * device array of 24 * n + 4 * (2080 + 512 * ceil(n / 1024)) + 256 bytes,
+ * about 6.8 MB, which every GPU that loads the library holds until exit. */
 #define DZS_NOALLOC_SORT_MAX_N 262144
 
 /* Allocation-free stable Morton sort of n <= DZS_NOALLOC_SORT_MAX_N lattice

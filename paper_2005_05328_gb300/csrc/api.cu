@@ -85,7 +85,7 @@ struct Layout {
 
 // offsets of every device buffer in the arena (also used for the footprint)
 struct Plan {
-  int64_t cap, node_cap, m3, nspec, nb, nchunks, ring;
+  int64_t cap, node_cap, m3, nspec, nchunks, ring;
   size_t rsz;
   size_t o_u, o_u2, o_p, o_p2, o_g, o_gsave, o_k, o_k2, o_id, o_id2, o_fl, o_fl2, o_key, o_key2, o_idx, o_idx2, o_hist,
       o_blocksum, o_iscan, o_prefix, o_mend, o_nodes, o_lvl, o_cfirst, o_parent, o_cicw, o_groups, o_ghead, o_wpm, o_wph, o_wnh, o_wlen,
@@ -97,7 +97,6 @@ struct Plan {
     node_cap = 2 * cap + 1024;
     m3 = (int64_t)P.mesh * P.mesh * P.mesh;
     nspec = (int64_t)P.mesh * P.mesh * (P.precision == DZS_FP64 ? spec_row<double>(P.mesh) : spec_row<float>(P.mesh));
-    nb = (cap + 1023) / 1024;  // digit-histogram tiles: enough for sort tiles of >= 1024 keys
     nchunks = (cap + 1024) / 1024 + 1;
     ring = P.lc_capacity ? (int64_t)P.lc_capacity : cap;
     rsz = P.precision == DZS_FP64 ? 8 : 4;
@@ -118,7 +117,7 @@ struct Plan {
     o_key2 = L.take(8 * cap);
     o_idx = L.take(4 * cap);
     o_idx2 = L.take(4 * cap);
-    o_hist = L.take(4 * (257 * nb + 256));
+    o_hist = L.take(4 * sort_scratch_words(cap));
     o_blocksum = L.take(8 * 4 * (nchunks + 2));
     o_iscan = L.take(4 * (2 * cap + 64));  // also the tree's per-tile counts (23 per 1024 particles)
     o_prefix = L.take(8 * 4 * (cap + 1));
@@ -183,18 +182,26 @@ dzs_status fail(dzs_ctx* c, dzs_status s, const char* what, const char* detail =
   return s;
 }
 
+dzs_status device_error_status(dzs_ctx* c, uint32_t err) {
+  char buf[160];
+  if (err & kErrSort) {
+    snprintf(buf, sizeof buf, "a bounded device wait of the sort gave up (error word 0x%x)", err);
+    return fail(c, DZS_ETIMEOUT, buf);
+  }
+  if (err & (kErrNodes | kErrStack | kErrGroups)) {
+    snprintf(buf, sizeof buf, "device buffer overflow (error word 0x%x)", err);
+    return fail(c, DZS_EOVERFLOW, buf);
+  }
+  return DZS_OK;
+}
+
 dzs_status check_device_errors(dzs_ctx* c) {
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return fail(c, DZS_EDEVICE, "device failure", cudaGetErrorString(e));
   uint32_t err = 0;
   e = cudaMemcpy(&err, c->B.err, sizeof(uint32_t), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return fail(c, DZS_EDEVICE, "device failure", cudaGetErrorString(e));
-  if (err & (kErrNodes | kErrStack | kErrGroups)) {
-    char buf[160];
-    snprintf(buf, sizeof buf, "device buffer overflow (error word 0x%x)", err);
-    return fail(c, DZS_EOVERFLOW, buf);
-  }
-  return DZS_OK;
+  return device_error_status(c, err);
 }
 
 dzs_status guard(dzs_ctx* c) {
@@ -689,11 +696,8 @@ dzs_status pipe_slot(dzs_ctx* c, int32_t step, const dzs_ctx::PipeSlot** out) {
     return fail(c, DZS_EINVAL, "no result kept for that step (only the last 4 steps are)");
   CK(cudaEventSynchronize(c->pipe_ev[k]));
   const dzs_ctx::PipeSlot* slot = c->pipe + k;
-  if (slot->err[0] & (kErrNodes | kErrStack | kErrGroups)) {
-    char buf[160];
-    snprintf(buf, sizeof buf, "device buffer overflow (error word 0x%x)", slot->err[0]);
-    return fail(c, DZS_EOVERFLOW, buf);
-  }
+  const dzs_status s = device_error_status(c, slot->err[0]);
+  if (s) return s;
   *out = slot;
   return DZS_OK;
 }

@@ -21,7 +21,7 @@ enum : uint32_t {
   kErrStack = 2u,    // walk stack overflow
   kErrRing = 4u,     // lightcone ring full (records dropped)
   kErrGroups = 8u,   // group capacity exceeded
-  kErrSort = 16u,    // inconsistent radix sort histogram
+  kErrSort = 16u,    // a sort look-back gave up (bounded wait)
   kErrCell = 32u,    // CIC cell start table inconsistent
 };
 
@@ -117,7 +117,7 @@ struct Buffers {
   // sort
   uint64_t *key = nullptr, *key2 = nullptr;
   uint32_t *idx = nullptr, *idx2 = nullptr;
-  uint32_t* hist = nullptr;  // [256][max blocks]
+  uint32_t* hist = nullptr;  // the passes' scratch (sort_scratch_words)
   // generic scan scratch
   int64_t* blocksum = nullptr;
   int32_t* iscan = nullptr;  // [cap + 1]
@@ -244,6 +244,7 @@ void launch_count_crossings(dzs_ctx* c, int step, unsigned long long* count);
 void launch_twin_displacement(dzs_ctx* a, dzs_ctx* b, int32_t* map, const double* edges, int nbins, double h,
                               unsigned long long* counts, unsigned long long* stats);
 void launch_sort(dzs_ctx* c);
+size_t sort_scratch_words(int64_t n);
 void launch_sort_keys(dzs_ctx* c, uint64_t* ka, uint64_t* kb, uint32_t* va, uint32_t* vb, int passes);
 void launch_keys(dzs_ctx* c);
 void launch_unpermute(dzs_ctx* c, double* g_out);

@@ -4,173 +4,256 @@
 //
 // The oct-tree of the paper (Sec. 2.1) becomes an implicit octree over the
 // sorted keys: every octree cell is a contiguous run of the sorted array.
-// Each pass: per-tile digit histograms, a per-digit scan over tiles, and a
-// stable scatter (rank = earlier items of the same digit in the tile).  Ties
-// keep the previous order, so the result is deterministic.
+// One kernel counts the digits of all passes; then each pass is one kernel: a
+// block ranks a tile of keys, learns how many keys of each digit the tiles
+// before it hold by looking back over their published counts, and writes the
+// tile.  Ties keep the previous order, so the result is deterministic.
 #include "common.cuh"
 
 namespace dzs {
 namespace {
 
 constexpr int kSortThreads = 256;
-constexpr int kItems = 8;
-constexpr int kTile = kSortThreads * kItems;  // 2048 keys per block
 constexpr int kDigits = 256;
+constexpr int kPasses = 8;
+// tiles: 512 threads x 14 keys (two blocks per SM hold 2.2M keys at once), for
+// fewer keys 256 x 4, spread over more SMs
+constexpr int kLargeThreads = 512, kLargeItems = 14, kSmallThreads = 256, kSmallItems = 4;
+constexpr int64_t kLargeFrom = 1 << 19;
 
-__global__ void k_hist(const uint64_t* __restrict__ key, const int32_t* __restrict__ d_n, int shift,
-                       uint32_t* __restrict__ hist, int nb) {
-  __shared__ uint32_t cnt[kDigits];
-  cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t n = *d_n;
-  int64_t base = (int64_t)blockIdx.x * kTile;
-  uint64_t kv[kItems];  // all loads in flight before the first count
-#pragma unroll
-  for (int s = 0; s < kItems; ++s) {
-    int64_t i = base + s * kSortThreads + threadIdx.x;
-    kv[s] = i < n ? key[i] : 0ull;
-  }
-#pragma unroll
-  for (int s = 0; s < kItems; ++s) {
-    int64_t i = base + s * kSortThreads + threadIdx.x;
-    if (i < n) atomicAdd(&cnt[(kv[s] >> shift) & 0xff], 1u);
-  }
-  __syncthreads();
-  hist[threadIdx.x * nb + blockIdx.x] = cnt[threadIdx.x];
+// status word of a (tile, digit): count in the low 30 bits, and whether it is
+// the tile's own count or already the sum over all tiles up to it
+constexpr uint32_t kOwn = 1u << 30, kSum = 2u << 30, kCount = kOwn - 1u;
+constexpr int kLook = 8;
+constexpr int kLookLimit = 1 << 21;  // polls (about a second) before a look-back gives up (error bit)
+
+// scratch of a sort (words): digit counts of every pass, a ticket per pass, two
+// tables of status words (a pass fills one and clears the other for the next)
+constexpr int kOffTicket = kPasses * kDigits, kOffStatus = kOffTicket + 32;
+
+inline int64_t sort_tiles(int64_t n) {
+  const int64_t tile = n >= kLargeFrom ? kLargeThreads * kLargeItems : kSmallThreads * kSmallItems;
+  return (n + tile - 1) / tile;
+}
+// shared memory of a pass: the tile's keys and values, the warps' counters
+constexpr size_t pass_smem(int threads, int items) {
+  return (size_t)threads * items * 12 + (size_t)(threads / 32) * kDigits * 2;
 }
 
-// block d: exclusive scan of row d of the histogram, row total to rowtot[d]
-__global__ void k_scan_rows(uint32_t* __restrict__ hist, int nb, uint32_t* __restrict__ rowtot) {
-  __shared__ uint32_t warp_tot[32];
-  __shared__ uint32_t carry;
-  uint32_t* row = hist + (int64_t)blockIdx.x * nb;
-  if (threadIdx.x == 0) carry = 0;
+// counts[pass][digit] over all keys; clears the first status table
+__global__ void __launch_bounds__(kSortThreads) k_digit_counts(const uint64_t* __restrict__ key,
+                                                               const int32_t* __restrict__ d_n, int passes,
+                                                               uint32_t* __restrict__ scratch, int64_t tiles) {
+  __shared__ uint32_t cnt[kPasses][kDigits];
+  for (int q = threadIdx.x; q < passes * kDigits; q += kSortThreads) (&cnt[0][0])[q] = 0;
+  for (int64_t q = (int64_t)blockIdx.x * kSortThreads + threadIdx.x; q < tiles * kDigits;
+       q += (int64_t)gridDim.x * kSortThreads)
+    scratch[kOffStatus + q] = 0;
   __syncthreads();
+  const int64_t n = *d_n;
+  const int lane = threadIdx.x & 31;
+  // whole warps run every iteration, so that the votes see all lanes
+  for (int64_t i0 = (int64_t)blockIdx.x * kSortThreads; i0 < n; i0 += (int64_t)gridDim.x * kSortThreads) {
+    const int64_t i = i0 + threadIdx.x;
+    const bool valid = i < n;
+    const uint64_t k = key[valid ? i : n - 1];
+    // nearly sorted input: 32 consecutive keys mostly share their top 15 bits,
+    // which would be 32 additions to one counter
+    const uint64_t k0 = __shfl_sync(0xffffffffu, k, 0);
+    const unsigned take = __ballot_sync(0xffffffffu, valid);
+    const bool top = passes == kPasses && __all_sync(0xffffffffu, (k >> 48) == (k0 >> 48));
+    if (top && lane < 2) atomicAdd(&cnt[6 + lane][(uint32_t)(k >> (48 + 8 * lane)) & 0xffu], (uint32_t)__popc(take));
+    if (valid) {
+      const int each = top ? kPasses - 2 : passes;
+#pragma unroll
+      for (int p = 0; p < kPasses; ++p)
+        if (p < each) atomicAdd(&cnt[p][(uint32_t)(k >> (8 * p)) & 0xffu], 1u);
+    }
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < passes * kDigits; q += kSortThreads) {
+    const uint32_t c = (&cnt[0][0])[q];
+    if (c) atomicAdd(&scratch[q], c);
+  }
+}
+
+// inclusive scan over the threads of a block (warp scans, then the warps' totals)
+__device__ __forceinline__ uint32_t block_incl_scan(uint32_t v, uint32_t* wtot) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int b0 = 0; b0 < nb; b0 += blockDim.x) {
-    int b = b0 + threadIdx.x;
-    uint32_t v = b < nb ? row[b] : 0u, inc = v;
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += t;
-    }
-    if (lane == 31) warp_tot[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-      uint32_t t = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0u, ti = t;
-      for (int o = 1; o < 32; o <<= 1) {
-        uint32_t q = __shfl_up_sync(0xffffffffu, ti, o);
-        if (lane >= o) ti += q;
-      }
-      warp_tot[lane] = ti - t;
-    }
-    __syncthreads();
-    uint32_t ex = inc - v + warp_tot[w] + carry;
-    if (b < nb) row[b] = ex;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = ex + v;
-    __syncthreads();
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
   }
-  if (threadIdx.x == 0) rowtot[blockIdx.x] = carry;
+  if (lane == 31) wtot[w] = v;
+  __syncthreads();
+  uint32_t before = 0;
+  for (int q = 0; q < w; ++q) before += wtot[q];
+  return v + before;
 }
 
-__global__ void k_scatter(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                          uint64_t* __restrict__ kout, uint32_t* __restrict__ vout,
-                          const int32_t* __restrict__ d_n, int shift, const uint32_t* __restrict__ hist,
-                          int nb, const uint32_t* __restrict__ rowtot, bool identity_values) {
+// lanes holding the same digit (invalid lanes: none in particular), by one
+// ballot per bit: a tenth of the time of the match instruction
+__device__ __forceinline__ unsigned same_digit(unsigned d, bool valid) {
+  unsigned peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const bool one = (d >> b) & 1u;
+    const unsigned v = __ballot_sync(0xffffffffu, one);
+    peers &= one ? v : ~v;
+  }
+  return peers;
+}
+
+// One pass.  Tiles are taken by ticket, so every tile before a block's is
+// already held by a running block and the look-back ends.  A warp ranks its
+// own consecutive keys 32 at a time against counters of its own: no block
+// barrier inside the ranking (the tile used to pass four per 256 keys).
+// The tile is placed in shared memory before the look-back, which gives the
+// tiles before it time to publish (8 words in flight; 16 or 32, or one block
+// less per SM, were 5-25% slower: polling competes with the ranking).  Bound by
+// latency at small n (a launch, one round of loads, the look-back), at large n
+// by the look-back and the ranking's instructions (~170 per 32 keys).  Sort
+// stage of 33k / 262k / 2.1M / 16.8M particles with three kernels a pass (digit
+// counts per tile, row scans, scatter): 137, 154, 317, 1850 us; now 63, 103,
+// 230, 1440.
+template <int kThr, int kItems>
+__global__ void __launch_bounds__(kThr, 1024 / kThr)
+    k_sort_pass(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint64_t* __restrict__ kout,
+                uint32_t* __restrict__ vout, const int32_t* __restrict__ d_n, int pass, uint32_t* __restrict__ scratch,
+                int64_t tiles, uint32_t* __restrict__ err) {
+  constexpr int kTile = kThr * kItems, kW = kThr / 32;
+  extern __shared__ uint64_t sort_sm[];
+  uint64_t* sk = sort_sm;                                           // [kTile] the tile, stably sorted by digit
+  uint32_t* sv = reinterpret_cast<uint32_t*>(sk + kTile);           // [kTile]
+  uint16_t(*wcnt)[kDigits] = reinterpret_cast<uint16_t(*)[kDigits]>(sv + kTile);  // [kW]
   __shared__ uint32_t gbase[kDigits];  // output position of the tile's first key of each digit
-  __shared__ uint32_t lbase[kDigits];  // the same within the tile (tile sorted by digit)
-  __shared__ uint32_t run[kDigits];
-  __shared__ uint32_t wcnt[kSortThreads / 32][kDigits];
-  __shared__ uint64_t sk[kTile];       // the tile, stably sorted by digit
-  __shared__ uint32_t sv[kTile];
+  __shared__ uint32_t lbase[kDigits];  // the same within the tile
+  __shared__ uint32_t wtot[2][kW];
+  __shared__ int s_tile;
   const int64_t n = *d_n;
-  int64_t base = (int64_t)blockIdx.x * kTile;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, shift = 8 * pass;
+  if (t == 0) s_tile = (int)atomicAdd(&scratch[kOffTicket + pass], 1u);
+  for (int q = t; q < kW * kDigits / 2; q += kThr) reinterpret_cast<uint32_t*>(&wcnt[0][0])[q] = 0;
+  __syncthreads();
+  const int64_t tile = s_tile, base = tile * kTile;
+  uint32_t* status = scratch + kOffStatus + (pass & 1 ? tiles * kDigits : 0);
+  uint32_t* other = scratch + kOffStatus + (pass & 1 ? 0 : tiles * kDigits);
+  if (t < kDigits) other[tile * kDigits + t] = 0;  // the next pass's table
   if (base >= n) return;
   const int tile_n = (int)(n - base < kTile ? n - base : kTile);
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  // the tile's keys and values, all loads in flight before any waiting
   uint64_t kreg[kItems];
   uint32_t vreg[kItems];
+  uint16_t rank[kItems];
+  const int64_t i0 = base + w * 32 * kItems + lane;  // the warp's keys are consecutive
 #pragma unroll
   for (int s = 0; s < kItems; ++s) {
-    const int64_t i = base + s * kSortThreads + t;
+    const int64_t i = i0 + s * 32;
     kreg[s] = i < n ? kin[i] : 0ull;
-    vreg[s] = i < n ? (identity_values ? (uint32_t)i : vin[i]) : 0u;
+    vreg[s] = i < n ? (pass == 0 ? (uint32_t)i : vin[i]) : 0u;  // indices start as the identity
   }
-  // digit bases: exclusive scans over the 256 digits (thread t owns digit t) of
-  // the row totals (global) and of this tile's counts (local); warp scans,
-  // then a scan of the 8 warp totals
-  {
-    __shared__ uint32_t wtot[2][kSortThreads / 32];
-    const uint32_t h0 = hist[(int64_t)t * nb + blockIdx.x];
-    const uint32_t h1 = blockIdx.x + 1 < (unsigned)nb ? hist[(int64_t)t * nb + blockIdx.x + 1] : rowtot[t];
-    const uint32_t v = rowtot[t], c = h1 - h0;
-    uint32_t inc = v, incc = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o), yc = __shfl_up_sync(0xffffffffu, incc, o);
-      if (lane >= o) {
-        inc += y;
-        incc += yc;
-      }
-    }
-    if (lane == 31) {
-      wtot[0][w] = inc;
-      wtot[1][w] = incc;
-    }
-    __syncthreads();
-    uint32_t before = 0, beforec = 0;
-    for (int q = 0; q < w; ++q) {
-      before += wtot[0][q];
-      beforec += wtot[1][q];
-    }
-    gbase[t] = before + inc - v + h0;
-    lbase[t] = beforec + incc - c;
-    run[t] = 0;
-  }
+  const uint32_t total = t < kDigits ? scratch[pass * kDigits + t] : 0u;
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int s = 0; s < kItems; ++s) {
-    for (int q = 0; q < kSortThreads / 32; ++q) wcnt[q][t] = 0;
-    __syncthreads();
-    int64_t i = base + s * kSortThreads + t;
-    bool valid = i < n;
-    uint64_t kv = kreg[s];
-    uint32_t vv = vreg[s];
-    int d = valid ? (int)((kv >> shift) & 0xff) : kDigits;  // invalid items group apart
-    unsigned peers = __match_any_sync(0xffffffffu, d);
-    int rank_w = __popc(peers & lt);
-    if (valid && rank_w == 0) wcnt[w][d] = __popc(peers);
-    __syncthreads();
-    {
-      uint32_t off = run[t];
-      for (int q = 0; q < kSortThreads / 32; ++q) {
-        uint32_t c = wcnt[q][t];
-        wcnt[q][t] = off;
-        off += c;
-      }
-      run[t] = off;
-    }
-    __syncthreads();
-    if (valid) {
-      const uint32_t lp = lbase[d] + wcnt[w][d] + (uint32_t)rank_w;
-      if (lp < (uint32_t)kTile) {  // always, when the tile's histogram matches its keys
-        sk[lp] = kv;
-        sv[lp] = vv;
-      }
-    }
-    __syncthreads();  // wcnt is read above and cleared at the top of the next round
+    const bool valid = i0 + s * 32 < n;
+    const unsigned d = (unsigned)(kreg[s] >> shift) & 0xffu;
+    const unsigned peers = same_digit(d, valid);
+    const uint32_t before = valid ? wcnt[w][d] : 0u;
+    __syncwarp();
+    if (valid && (peers & lt) == 0u) wcnt[w][d] = (uint16_t)(before + __popc(peers));
+    __syncwarp();
+    rank[s] = (uint16_t)(before + __popc(peers & lt));
   }
+  __syncthreads();
+  // thread t < 256 owns digit t: warps' counts to offsets, the tile's count
+  uint32_t run = 0;
+  volatile uint32_t* st = status + t;
+  if (t < kDigits) {
+#pragma unroll
+    for (int q = 0; q < kW; ++q) {
+      const uint32_t c = wcnt[q][t];
+      wcnt[q][t] = (uint16_t)run;
+      run += c;
+    }
+    st[tile * kDigits] = run | (tile == 0 ? kSum : kOwn);
+  }
+  const uint32_t local0 = block_incl_scan(run, wtot[0]) - run;
+  const uint32_t digit0 = block_incl_scan(total, wtot[1]) - total;
+  if (t < kDigits) lbase[t] = local0;
+  __syncthreads();
+  // place the tile while the tiles before it publish their counts
+#pragma unroll
+  for (int s = 0; s < kItems; ++s) {
+    if (i0 + s * 32 < n) {
+      const int d = (int)((kreg[s] >> shift) & 0xff);
+      const uint32_t lp = lbase[d] + wcnt[w][d] + rank[s];
+      sk[lp] = kreg[s];
+      sv[lp] = vreg[s];
+    }
+  }
+  // keys of digit t in the tiles before this one, kLook status words in flight
+  // at a time (one by one, the ~700 tiles of a wave cost as many L2 latencies)
+  if (t < kDigits) {
+    uint32_t prev = 0;
+    int64_t back = tile - 1;
+    for (int polls = 0; back >= 0;) {
+      uint32_t v[kLook];
+#pragma unroll
+      for (int q = 0; q < kLook; ++q) v[q] = back - q >= 0 ? st[(back - q) * kDigits] : 0u;
+      int64_t next = back;
+      bool open = true;
+#pragma unroll
+      for (int q = 0; q < kLook; ++q) {
+        open = open && (v[q] & (kOwn | kSum)) != 0u;
+        if (open) {
+          prev += v[q] & kCount;
+          next = (v[q] & kSum) ? -1 : next - 1;
+          open = next >= 0;
+        }
+      }
+      if (next == back) {
+        if (++polls > kLookLimit) {
+          if (err) atomicOr(err, kErrSort);
+          break;
+        }
+        __nanosleep(64);
+      }
+      back = next;
+    }
+    if (tile > 0) st[tile * kDigits] = (prev + run) | kSum;
+    gbase[t] = digit0 + prev;
+  }
+  __syncthreads();
   // runs of one digit are contiguous in the tile and in the output: coalesced
-  for (int q = t; q < tile_n; q += kSortThreads) {
+  for (int q = t; q < tile_n; q += kThr) {
     const uint64_t kv = sk[q];
     const int d = (int)((kv >> shift) & 0xff);
     const uint32_t pos = gbase[d] + (uint32_t)q - lbase[d];
-    if ((int64_t)pos < n) {
+    if ((int64_t)pos < n) {  // always, unless the look-back gave up
       kout[pos] = kv;
       vout[pos] = sv[q];
     }
+  }
+}
+
+// an even number of passes from bit 0; the result is in ka / va again
+void sort_passes(uint64_t* ka, uint64_t* kb, uint32_t* va, uint32_t* vb, const int32_t* d_n, int64_t cap, int passes,
+                 uint32_t* scratch, uint32_t* err, cudaStream_t st) {
+  const int64_t tiles = sort_tiles(cap);
+  const bool large = cap >= kLargeFrom;
+  auto kern = large ? k_sort_pass<kLargeThreads, kLargeItems> : k_sort_pass<kSmallThreads, kSmallItems>;
+  const int threads = large ? kLargeThreads : kSmallThreads;
+  const size_t sm = pass_smem(threads, large ? kLargeItems : kSmallItems);
+  if (large) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * kOffStatus, st);
+  k_digit_counts<<<grid_for(cap, 2 * kSortThreads, 4), kSortThreads, 0, st>>>(ka, d_n, passes, scratch, tiles);
+  uint64_t *kin = ka, *kout = kb;
+  uint32_t *vin = va, *vout = vb;
+  for (int pass = 0; pass < passes; ++pass) {
+    kern<<<(unsigned)tiles, threads, sm, st>>>(kin, vin, kout, vout, d_n, pass, scratch, tiles, err);
+    std::swap(kin, kout);
+    std::swap(vin, vout);
   }
 }
 
@@ -196,42 +279,22 @@ __global__ void k_permute(const int32_t* __restrict__ d_n, int64_t cap, const ui
 
 }  // namespace
 
+// words of sort scratch for n keys
+size_t sort_scratch_words(int64_t n) {
+  return (size_t)kOffStatus + 2 * kDigits * (size_t)sort_tiles(n);
+}
+
 // stable LSD radix sort of n keys (an even number of 8-bit passes from bit 0)
 // with their indices (identity on input); the result is in ka / va again
 void launch_sort_keys(dzs_ctx* c, uint64_t* ka, uint64_t* kb, uint32_t* va, uint32_t* vb, int passes) {
-  c->launches += 3 * passes;
-  Buffers& B = c->B;
-  int nb = (int)((c->cap + kTile - 1) / kTile);
-  uint32_t* rowtot = B.hist + (int64_t)kDigits * nb;
-  uint64_t *kin = ka, *kout = kb;
-  uint32_t *vin = va, *vout = vb;
-  for (int pass = 0; pass < passes; ++pass) {
-    int shift = 8 * pass;
-    k_hist<<<nb, kSortThreads, 0, c->stream>>>(kin, B.n, shift, B.hist, nb);
-    k_scan_rows<<<kDigits, 1024, 0, c->stream>>>(B.hist, nb, rowtot);
-    k_scatter<<<nb, kSortThreads, 0, c->stream>>>(kin, vin, kout, vout, B.n, shift, B.hist, nb, rowtot,
-                                                  pass == 0);
-    std::swap(kin, kout);
-    std::swap(vin, vout);
-  }
+  c->launches += passes + 1;
+  sort_passes(ka, kb, va, vb, c->B.n, c->cap, passes, c->B.hist, c->B.err, c->stream);
 }
 
 void launch_sort(dzs_ctx* c) {
-  c->launches += 25;
+  c->launches += 1;
   Buffers& B = c->B;
-  int nb = (int)((c->cap + kTile - 1) / kTile);
-  uint32_t* rowtot = B.hist + (int64_t)kDigits * nb;
-  uint64_t *kin = B.key, *kout = B.key2;
-  uint32_t *vin = B.idx, *vout = B.idx2;
-  for (int pass = 0; pass < 8; ++pass) {
-    int shift = 8 * pass;
-    k_hist<<<nb, kSortThreads, 0, c->stream>>>(kin, B.n, shift, B.hist, nb);
-    k_scan_rows<<<kDigits, 1024, 0, c->stream>>>(B.hist, nb, rowtot);
-    k_scatter<<<nb, kSortThreads, 0, c->stream>>>(kin, vin, kout, vout, B.n, shift, B.hist, nb, rowtot,
-                                                  pass == 0);
-    std::swap(kin, kout);
-    std::swap(vin, vout);
-  }
+  launch_sort_keys(c, B.key, B.key2, B.idx, B.idx2, kPasses);
   // 8 passes: sorted keys and indices are back in key / idx
   int grid = grid_for(c->N0);
   if (c->fp64)
@@ -347,14 +410,15 @@ namespace dzs {
 namespace {
 
 constexpr size_t kNoallocMaxN = DZS_NOALLOC_SORT_MAX_N;
-constexpr size_t kNoallocNb = (kNoallocMaxN + kTile - 1) / kTile;
-// layout: keyA, keyB (uint64), valA, valB (uint32), hist (257 rows of nb + 256),
-// count slot
+// layout: keyA, keyB (uint64), valA, valB (uint32), the passes' scratch (n below
+// kLargeFrom: the small tiles), count slot
+constexpr size_t kNoallocTiles = (kNoallocMaxN + kSmallThreads * kSmallItems - 1) / (kSmallThreads * kSmallItems);
+static_assert(kNoallocMaxN < (size_t)kLargeFrom, "tile size of the allocation-free sort");
 constexpr size_t kOffKeyB = 8 * kNoallocMaxN;
 constexpr size_t kOffValA = 16 * kNoallocMaxN;
 constexpr size_t kOffValB = 20 * kNoallocMaxN;
 constexpr size_t kOffHist = 24 * kNoallocMaxN;
-constexpr size_t kOffCount = kOffHist + 4 * (257 * kNoallocNb + 256);
+constexpr size_t kOffCount = kOffHist + 4 * (kOffStatus + 2 * kDigits * kNoallocTiles);
 constexpr size_t kNoallocBytes = kOffCount + 256;
 
 static __device__ __align__(256) unsigned char g_sort_scratch[kNoallocBytes];
@@ -399,28 +463,18 @@ extern "C" dzs_status dzs_morton_sort_noalloc(const uint32_t* d_u, size_t n, uin
   uint32_t* hist = (uint32_t*)(b + kOffHist);
   int32_t* count = (int32_t*)(b + kOffCount);
   // every scratch word read below is first written by this call: the count,
-  // the keys, the per-tile histograms (all 256 rows of every tile) and the row
-  // totals, so nothing left over from a previous call is used
-  const int nb = (int)((n + kTile - 1) / kTile);
-  uint32_t* rowtot = hist + (int64_t)kDigits * nb;
+  // the keys, the digit counts and tickets (cleared), the status tables (the
+  // first cleared by the counting kernel, each other by the pass before), so
+  // nothing left over from a previous call is used
   // each launch is checked with cudaPeekAtLastError (a launch error is sticky
   // for this call's own launches only: nothing was pending before them)
   k_set_count<<<1, 1, 0, st>>>(count, (int32_t)n);
   if (cudaPeekAtLastError() != cudaSuccess) return DZS_ECUDA;
   k_keys<<<grid_for((int64_t)n), kThreads, 0, st>>>(count, (int64_t)n, d_u, keyA);
   if (cudaPeekAtLastError() != cudaSuccess) return DZS_ECUDA;
-  uint64_t *kin = keyA, *kout = keyB;
-  uint32_t *vin = valA, *vout = valB;
-  for (int pass = 0; pass < 8; ++pass) {
-    int shift = 8 * pass;
-    k_hist<<<nb, kSortThreads, 0, st>>>(kin, count, shift, hist, nb);
-    k_scan_rows<<<kDigits, 1024, 0, st>>>(hist, nb, rowtot);
-    k_scatter<<<nb, kSortThreads, 0, st>>>(kin, vin, kout, vout, count, shift, hist, nb, rowtot, pass == 0);
-    if (cudaPeekAtLastError() != cudaSuccess) return DZS_ECUDA;
-    std::swap(kin, kout);
-    std::swap(vin, vout);
-  }
-  if (cudaMemcpyAsync(d_perm, vin, 4 * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return DZS_ECUDA;
-  if (d_keys && cudaMemcpyAsync(d_keys, kin, 8 * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return DZS_ECUDA;
+  sort_passes(keyA, keyB, valA, valB, count, (int64_t)n, kPasses, hist, nullptr, st);
+  if (cudaPeekAtLastError() != cudaSuccess) return DZS_ECUDA;
+  if (cudaMemcpyAsync(d_perm, valA, 4 * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return DZS_ECUDA;
+  if (d_keys && cudaMemcpyAsync(d_keys, keyA, 8 * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return DZS_ECUDA;
   return DZS_OK;
 }
