@@ -175,7 +175,8 @@ struct dzs_ctx {
   cudaStream_t stream = nullptr;
   bool fp64 = false;
   int64_t N0 = 0, cap = 0, node_cap = 0;
-  int M = 0, logM = 0, n1 = 0;  // logM: depth of the Morton cell table (floor log2 M)
+  int M = 0, logM = 0, n1 = 0;  // logM: floor log2 M
+  int cell_depth = 0;            // depth of the Morton cell table (tree, PM tiles)
   bool mesh_pow2 = true;         // false: M = 3 2^a, deposited through a row-major cell sort
   int sort_blocks = 0;
   double lat = 0, scale = 0, gm0 = 0, eps0 = 0, rs = 0, rcut = 0, rcut_lat2 = 0;
@@ -232,6 +233,18 @@ struct dzs_ctx {
 };
 
 namespace dzs {
+
+// meshes whose CIC deposit and interpolation run on 16-wide tiles straight from
+// the particles (pm.cu): FP32, M = 2^m from 128 on (512 tiles), and less than
+// half a particle a cell on average.  Elsewhere per-cell weight records and
+// node gradients are shared by enough particles to be worth their own pass
+// (256^3 on mesh 256: PM stage 0.64 ms, with the tiles 1.13), the tiles are too
+// few (32^3 on mesh 64), or FP64 arithmetic is the bound (64^3 on mesh 128: 161
+// us, with the tiles 178).  Mesh = 2 n1d, FP32: 128^3 early 0.38 -> 0.24, late
+// 0.30 -> 0.16, 256^3 2.92 -> 1.77 ms with the tiles.
+inline bool tile_mesh(const dzs_ctx* c) {
+  return !c->fp64 && c->mesh_pow2 && c->M >= 128 && 2 * c->N0 < (int64_t)c->M * c->M * c->M;
+}
 
 // host-side cosmology (host.cu)
 void compute_tables(const dzs_params& P, Tables& T);

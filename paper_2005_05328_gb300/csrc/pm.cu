@@ -89,10 +89,126 @@ __device__ __forceinline__ void store8(R* __restrict__ dst, const R (&v)[8]) {
   }
 }
 
+// corner weight sums of one cell: acc[o] = sum over the cell's particles, in
+// order, of k w_o, w_o the CIC weight of the cell's corner node o = (ox, oy, oz)
+template <class R>
+__device__ __forceinline__ void add_corners(uint32_t ux, uint32_t uy, uint32_t uz, uint32_t k, int M, R (&acc)[8]) {
+  const R fx = frac32<R>((uint32_t)((uint64_t)ux * (uint64_t)M)), fy = frac32<R>((uint32_t)((uint64_t)uy * (uint64_t)M)),
+          fz = frac32<R>((uint32_t)((uint64_t)uz * (uint64_t)M));
+  const R kk = (R)k;
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    const int ox = (o >> 2) & 1, oy = (o >> 1) & 1, oz = o & 1;
+    acc[o] += kk * ((ox ? fx : (R)1 - fx) * (oy ? fy : (R)1 - fy) * (oz ? fz : (R)1 - fz));
+  }
+}
+
+// M = 2^m: density contrast of one 16^3 tile of nodes per block.  Mesh cells are
+// Morton cells, so the tile's own particles are one contiguous run, those of its
+// lower neighbours' 8^3 cells 19 more; start is the table of Morton cells (2^sh9 per 8^3 cells).  The particle that
+// opens a cell sums the cell's corner weights in registers; the block then adds
+// corner o = 0..7 in turn, one barrier apart: the cells of a batch differ, so no
+// two threads add to a node at once and the order is fixed (deterministic).
+// Bound by latency: a tile is a few rounds of dependent loads.  It replaces a
+// pass that wrote each cell's sums to memory and a gather that read the bounds
+// of 729 cells and 8 records a node for each 8^3 tile: 177 + 29 (a finer cell
+// table) -> 145 us for 128^3 on mesh 256.
+constexpr int kCicThreads = 512;
+constexpr int kT = 16;  // nodes per side of a tile
+template <class R>
+__global__ void __launch_bounds__(kCicThreads) k_cic_tile(const int32_t* __restrict__ start, int sh9,
+                                                          const int32_t* __restrict__ d_n, int64_t cap,
+                                                          const uint64_t* __restrict__ key, int sh,
+                                                          const uint32_t* __restrict__ u, const uint32_t* __restrict__ k,
+                                                          int M, R* __restrict__ delta, R inv_nbar) {
+  constexpr int S = kT / 8, E = S + 1, kRuns = E * E * E;  // 8^3 cells per axis with the lower neighbour
+  __shared__ R acc[kT * kT * kT];
+  __shared__ int32_t first[32], upto[32];  // runs of the neighbours' cells, running totals (0 for the own ones)
+  const int T = M / kT, T8 = M >> 3, tile = blockIdx.x;
+  const int tx = tile / (T * T), ty = (tile / T) % T, tz = tile % T;
+  const int64_t n = *d_n;
+  auto cell8 = [](uint32_t x, uint32_t y, uint32_t z) {
+    return (int64_t)((spread3(x) << 2) | (spread3(y) << 1) | spread3(z));
+  };
+  const int64_t own8 = cell8((uint32_t)(tx * S), (uint32_t)(ty * S), (uint32_t)(tz * S));
+  const int32_t p0 = start[own8 << sh9], p1 = start[(own8 + S * S * S) << sh9];
+  if (threadIdx.x < 32) {
+    const int o = threadIdx.x;  // (x, y, z) offset + 1 per axis
+    const int ox = o / (E * E), oy = (o / E) % E, oz = o % E;
+    int32_t s = 0, len = 0;
+    if (o < kRuns && (ox == 0 || oy == 0 || oz == 0)) {
+      const int64_t c = cell8((uint32_t)(tx * S + ox - 1 + T8) % (uint32_t)T8, (uint32_t)(ty * S + oy - 1 + T8) % (uint32_t)T8,
+                              (uint32_t)(tz * S + oz - 1 + T8) % (uint32_t)T8);
+      s = start[c << sh9];
+      len = start[(c + 1) << sh9] - s;
+    }
+#pragma unroll
+    for (int q = 1; q < 32; q <<= 1) {
+      const int32_t v = __shfl_up_sync(0xffffffffu, len, q);
+      if (o >= q) len += v;
+    }
+    first[o] = s;
+    upto[o] = len;
+  }
+  for (int q = threadIdx.x; q < kT * kT * kT; q += kCicThreads) acc[q] = (R)0;
+  __syncthreads();
+  const int own = p1 - p0, total = own + upto[31];
+  for (int t0 = 0; t0 < total; t0 += kCicThreads) {
+    // the thread's cell: its lowest corner node in tile coordinates (-1: below)
+    int x = 0, y = 0, z = 0;
+    bool take = false;
+    R w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const int t = t0 + (int)threadIdx.x;
+    if (t < total) {
+      int64_t i = (int64_t)p0 + t;
+      int ox = 1, oy = 1, oz = 1;
+      if (t >= own) {
+        const int v = t - own;
+        int o = 0;
+#pragma unroll
+        for (int step = 16; step >= 1; step >>= 1)
+          if (upto[o + step - 1] <= v) o += step;
+        i = (int64_t)first[o] + v - (o > 0 ? upto[o - 1] : 0);
+        ox = o / (E * E);
+        oy = (o / E) % E;
+        oz = o % E;
+      }
+      const uint64_t c = key[i] >> sh;
+      const bool opens = i == 0 || (key[i - 1] >> sh) != c;
+      const int mo = (int)c & (kT * kT * kT - 1);
+      x = ((mo >> 6) & 4) | ((mo >> 4) & 2) | ((mo >> 2) & 1);
+      y = ((mo >> 5) & 4) | ((mo >> 3) & 2) | ((mo >> 1) & 1);
+      z = ((mo >> 4) & 4) | ((mo >> 2) & 2) | (mo & 1);
+      x |= (mo >> 8) & 8;
+      y |= (mo >> 7) & 8;
+      z |= (mo >> 6) & 8;
+      // a lower neighbour's cell counts when it touches the tile: its last layer
+      take = opens && (ox > 0 || (x & 7) == 7) && (oy > 0 || (y & 7) == 7) && (oz > 0 || (z & 7) == 7);
+      if (ox == 0) x = -1;
+      if (oy == 0) y = -1;
+      if (oz == 0) z = -1;
+      if (take)
+        for (int64_t j = i; j < n && (j == i || (key[j] >> sh) == c); ++j)
+          add_corners<R>(u[j], u[cap + j], u[2 * cap + j], k[j], M, w);
+    }
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      const int ax = x + (o >> 2), ay = y + ((o >> 1) & 1), az = z + (o & 1);
+      if (take && (unsigned)ax < (unsigned)kT && (unsigned)ay < (unsigned)kT && (unsigned)az < (unsigned)kT)
+        acc[(ax * kT + ay) * kT + az] += w[o];
+      __syncthreads();
+    }
+  }
+  for (int t = threadIdx.x; t < kT * kT * kT; t += kCicThreads) {
+    const int a = t / (kT * kT), b = (t / kT) % kT, c = t % kT;
+    delta[((int64_t)(tx * kT + a) * M + (ty * kT + b)) * M + (tz * kT + c)] = acc[t] * inv_nbar - (R)1;
+  }
+}
+
 // W[8 i + o], i the first particle of a cell = sum over the cell's particles,
 // in order, of k w_o, w_o the CIC weight of the cell's corner node
-// o = (ox, oy, oz): each particle's weights are computed once (not once per
-// node that reads it); the 8 sums of a cell are one aligned 8-value record
+// o = (ox, oy, oz); the 8 sums of a cell are one aligned 8-value record.  For the
+// meshes tile_mesh leaves out.
 template <class R>
 __global__ void k_cic_cellw(const int32_t* __restrict__ d_n, int64_t cap, const uint64_t* __restrict__ key, int sh,
                             const uint32_t* __restrict__ u, const uint32_t* __restrict__ k, int M,
@@ -102,24 +218,14 @@ __global__ void k_cic_cellw(const int32_t* __restrict__ d_n, int64_t cap, const 
     const uint64_t c = key[i] >> sh;
     if (i > 0 && (key[i - 1] >> sh) == c) continue;  // not the first of its cell
     R acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int64_t j = i; j < n && (key[j] >> sh) == c; ++j) {
-      R fx = frac32<R>((uint32_t)((uint64_t)u[j] * (uint64_t)M));
-      R fy = frac32<R>((uint32_t)((uint64_t)u[cap + j] * (uint64_t)M));
-      R fz = frac32<R>((uint32_t)((uint64_t)u[2 * cap + j] * (uint64_t)M));
-      const R kk = (R)k[j];
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        const int ox = (o >> 2) & 1, oy = (o >> 1) & 1, oz = o & 1;
-        acc[o] += kk * ((ox ? fx : (R)1 - fx) * (oy ? fy : (R)1 - fy) * (oz ? fz : (R)1 - fz));
-      }
-    }
+    for (int64_t j = i; j < n && (key[j] >> sh) == c; ++j)
+      add_corners<R>(u[j], u[cap + j], u[2 * cap + j], k[j], M, acc);
     store8(W + 8 * i, acc);
   }
 }
 
-// the same for a mesh of M = 3 2^a: particles visited in row-major cell order
-// through the cell sort (sorted cell keys ck, original indices perm); W is
-// indexed by the sorted position of a cell's first particle
+// the same for M = 3 2^a, at sorted positions t: particles visited in row-major cell order through the
+// cell sort (sorted cell keys ck, original indices perm)
 template <class R>
 __global__ void k_cic_cellw_perm(const int32_t* __restrict__ d_n, int64_t cap, const uint64_t* __restrict__ ck,
                                  const uint32_t* __restrict__ perm, const uint32_t* __restrict__ u,
@@ -131,15 +237,7 @@ __global__ void k_cic_cellw_perm(const int32_t* __restrict__ d_n, int64_t cap, c
     R acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (int64_t s = t; s < n && ck[s] == c; ++s) {
       const int64_t j = perm[s];
-      R fx = frac32<R>((uint32_t)((uint64_t)u[j] * (uint64_t)M));
-      R fy = frac32<R>((uint32_t)((uint64_t)u[cap + j] * (uint64_t)M));
-      R fz = frac32<R>((uint32_t)((uint64_t)u[2 * cap + j] * (uint64_t)M));
-      const R kk = (R)k[j];
-#pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        const int ox = (o >> 2) & 1, oy = (o >> 1) & 1, oz = o & 1;
-        acc[o] += kk * ((ox ? fx : (R)1 - fx) * (oy ? fy : (R)1 - fy) * (oz ? fz : (R)1 - fz));
-      }
+      add_corners<R>(u[j], u[cap + j], u[2 * cap + j], k[j], M, acc);
     }
     store8(W + 8 * t, acc);
   }
@@ -269,15 +367,77 @@ __global__ void k_pm_interp(const int32_t* __restrict__ d_n, int64_t cap, const 
   }
 }
 
-// g = -grad phi (four-point stencil at the 8 surrounding nodes), CIC weights.
-// One block per 8^3 tile of cells = one depth-(m-3) octree cell, whose
-// particles are one contiguous Morton run.  The block stages the 13^3 nodes of
-// phi the tile's stencils reach as 169 rows of 16 (z from bz - 4, aligned
-// 16-byte loads away from the periodic z edge), then either forms the
-// gradient at the 9^3 corner nodes once (many particles) or lets each
-// particle form its 8 corner gradients from the staged phi (few particles);
-// both use the same four-point formula, so the result does not depend on the
-// choice.
+// g = -grad phi (four-point stencil at the 8 surrounding nodes), CIC weights,
+// for M = 2^m.  One block per 8 x 16 x 16 tile of cells: four 8^3 octree cells that share their parent's x half, whose particles are
+// one contiguous Morton run.  The block stages the nodes of phi the tile's
+// stencils reach, 13 x 21 rows of 24 (z from bz - 4: aligned 16-byte
+// loads, which never straddle the periodic edge), then each particle reads its
+// 56 nodes.  Along an axis the two corners' stencils and weights make one
+// 6-point filter, so a component takes 4 x 6 multiply-adds; forming the
+// gradient at all corner nodes first cost a barrier and 9 KB more shared memory.
+// Bound by latency (staging, then reading the particles) and L2 bandwidth: the
+// 16-wide tile stages 3.2 nodes a cell, an 8-wide one 5.3.  128^3 on mesh 256:
+// 200 -> 90 us.
+constexpr int kInterpThreads = 256;
+constexpr int kTy = 16;  // cells per side of a tile along y and z
+template <class R>
+__global__ void __launch_bounds__(kInterpThreads) k_pm_interp_tile(const int32_t* __restrict__ start, int sh9,
+                                                                   int64_t cap, const uint32_t* __restrict__ u,
+                                                                   const R* __restrict__ phi, int M, R inv12dx,
+                                                                   R* __restrict__ g) {
+  constexpr int RY = kTy + 5, RZ = kTy + 8, kSub = kTy / 8;
+  extern __shared__ unsigned char pi_raw[];
+  R* ph = reinterpret_cast<R*>(pi_raw);  // [13][RY][RZ]: node (bx - 2 + i, by - 2 + j, bz - 4 + l)
+  const int T = M / kTy, tile = blockIdx.x;
+  const int tx = tile / (T * T), ty = (tile / T) % T, tz = tile % T;
+  const int bx = tx * 8, by = ty * kTy, bz = tz * kTy;
+  // depth m - 3 Morton cells tx, ty kSub .., tz kSub ..: consecutive from the first
+  const int64_t tp = (int64_t)((spread3((uint32_t)tx) << 2) | (spread3((uint32_t)(ty * kSub)) << 1) |
+                               spread3((uint32_t)(tz * kSub)));
+  const int32_t p0 = start[tp << sh9], p1 = start[(tp + kSub * kSub) << sh9];
+  if (p1 <= p0) return;  // empty tile (uniform across the block)
+  const int mask = M - 1;
+  using V = typename Vec16<R>::T;
+  constexpr int N = Vec16<R>::N, PER = RZ / N;  // vectors per row
+  for (int v = threadIdx.x; v < 13 * RY * PER; v += kInterpThreads) {
+    const int r = v / PER, q = v % PER, i = r / RY, j = r % RY;
+    const int64_t row = ((int64_t)((bx - 2 + i) & mask) * M + ((by - 2 + j) & mask)) * M;
+    reinterpret_cast<V*>(ph + r * RZ)[q] = *reinterpret_cast<const V*>(phi + row + ((bz - 4 + q * N) & mask));
+  }
+  __syncthreads();
+  for (int64_t i = p0 + threadIdx.x; i < p1; i += kInterpThreads) {
+    const uint64_t sx = (uint64_t)u[i] * (uint64_t)M, sy = (uint64_t)u[cap + i] * (uint64_t)M,
+                   sz = (uint64_t)u[2 * cap + i] * (uint64_t)M;
+    // inside the tile by construction (the particle lies in it); clamped all the same
+    const int cx = min(max((int)(sx >> 32) - bx, 0), 7), cy = min(max((int)(sy >> 32) - by, 0), kTy - 1),
+              cz = min(max((int)(sz >> 32) - bz, 0), kTy - 1);
+    const R fx = frac32<R>((uint32_t)sx), fy = frac32<R>((uint32_t)sy), fz = frac32<R>((uint32_t)sz);
+    const R wx[2] = {(R)1 - fx, fx}, wy[2] = {(R)1 - fy, fy}, wz[2] = {(R)1 - fz, fz};
+    const R* c = ph + ((cx + 2) * RY + cy + 2) * RZ + cz + 4;
+    auto six = [](const R (&w)[2], R m2, R m1, R z0, R z1, R q2, R q3) {
+      // w0 (8 (z1 - m1) - (q2 - m2)) + w1 (8 (q2 - z0) - (q3 - m1))
+      return w[0] * ((R)8 * (z1 - m1) - (q2 - m2)) + w[1] * ((R)8 * (q2 - z0) - (q3 - m1));
+    };
+    constexpr int SX = RY * RZ, SY = RZ;
+    R ax = 0, ay = 0, az = 0;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const R *lx = c + a * SY + b, *ly = c + a * SX + b, *lz = c + a * SX + b * SY;
+        ax += wy[a] * wz[b] * six(wx, lx[-2 * SX], lx[-SX], lx[0], lx[SX], lx[2 * SX], lx[3 * SX]);
+        ay += wx[a] * wz[b] * six(wy, ly[-2 * SY], ly[-SY], ly[0], ly[SY], ly[2 * SY], ly[3 * SY]);
+        az += wx[a] * wy[b] * six(wz, lz[-2], lz[-1], lz[0], lz[1], lz[2], lz[3]);
+      }
+    g[i] = -ax * inv12dx;
+    g[cap + i] = -ay * inv12dx;
+    g[2 * cap + i] = -az * inv12dx;
+  }
+}
+
+// the same for the meshes tile_mesh leaves out: one block per 8^3 tile forms the
+// gradient at the 9^3 corner nodes once for all its particles (tiles with fewer
+// than kFlyMax let each particle form its 8 corner gradients).
 constexpr int kFlyMax = 96;  // below this many particles a tile skips the node gradients
 
 template <class R>
@@ -291,9 +451,9 @@ __device__ __forceinline__ void grad_at(const R* __restrict__ ph, int i, int j, 
 }
 
 template <class R>
-__global__ void __launch_bounds__(128) k_pm_interp_tile(const int32_t* __restrict__ start, int64_t cap,
-                                                        const uint32_t* __restrict__ u, const R* __restrict__ phi,
-                                                        int M, R inv12dx, R* __restrict__ g) {
+__global__ void __launch_bounds__(128) k_pm_interp_nodes(const int32_t* __restrict__ start, int sh9, int64_t cap,
+                                                         const uint32_t* __restrict__ u, const R* __restrict__ phi,
+                                                         int M, R inv12dx, R* __restrict__ g) {
   extern __shared__ unsigned char pi_raw[];
   R* ph = reinterpret_cast<R*>(pi_raw);  // [169][16]: row (i, j) = node (bx - 2 + i, by - 2 + j), z = bz - 4 + slot
   R* gr = ph + 169 * 16;                 // [3][9][9][9], corner node (bx + i, ...)
@@ -303,7 +463,7 @@ __global__ void __launch_bounds__(128) k_pm_interp_tile(const int32_t* __restric
   const int bx = tx * 8, by = ty * 8, bz = tz * 8;
   // the tile's particles: Morton prefix of the tile at depth m - 3
   const uint32_t tp = (uint32_t)((spread3((uint32_t)tx) << 2) | (spread3((uint32_t)ty) << 1) | spread3((uint32_t)tz));
-  const int32_t p0 = start[(int64_t)tp << 9], p1 = start[((int64_t)tp + 1) << 9];
+  const int32_t p0 = start[(int64_t)tp << sh9], p1 = start[((int64_t)tp + 1) << sh9];
   if (p1 <= p0) return;  // empty tile (uniform across the block)
   const int mask = M - 1;
   if (bz >= 8 && bz + 16 <= M) {
@@ -364,7 +524,8 @@ __global__ void __launch_bounds__(128) k_pm_interp_tile(const int32_t* __restric
   }
 }
 
-// the deposit reads the depth-m cell table the tree build wrote for the same keys
+// the deposit finds its tiles' particles in the cell table the tree build wrote
+// for the same keys (table cells per 8^3 tile: 2^sh9)
 template <class R>
 void pm_deposit(dzs_ctx* c) {
   Buffers& B = c->B;
@@ -373,8 +534,13 @@ void pm_deposit(dzs_ctx* c) {
   double n0 = (double)c->N0;
   R inv_nbar = (R)((double)m3 / n0);
   if (c->mesh_pow2) {
-    // mesh cells are the depth-m Morton cells of the tree's table
-    const int sh = 3 * (kMaxLevel - c->logM);
+    const int sh9 = 3 * (c->cell_depth - c->logM + 3), sh = 3 * (kMaxLevel - c->logM);
+    if (sizeof(R) == 4 && tile_mesh(c)) {
+      k_cic_tile<float><<<(unsigned)(m3 / (kT * kT * kT)), kCicThreads, 0, c->stream>>>(
+          B.cell_start, sh9, B.n, c->cap, B.key, sh, B.u, B.k, M, (float*)B.rho, (float)inv_nbar);
+      return;
+    }
+    // the table's cells are the mesh's
     k_cic_cellw<R><<<grid_for(c->N0), kThreads, 0, c->stream>>>(B.n, c->cap, B.key, sh, B.u, B.k, M, (R*)B.cicw);
     k_cic_gather<R, true><<<(unsigned)(m3 / 512), 256, gather_smem<R>(), c->stream>>>(
         B.cell_start, B.n, (const R*)B.cicw, M, (R*)B.rho, inv_nbar);
@@ -415,12 +581,15 @@ void pm_interp(dzs_ctx* c) {
                                                                 (R*)B.g);
     return;
   }
-  const int64_t tiles = (int64_t)(M / 8) * (M / 8) * (M / 8);
-  const size_t sm = (169 * 16 + 3 * 729) * sizeof(R);
-  // 128 threads: a tile holds ~64 particles at the mean density, and smaller
-  // blocks keep more tiles' staging loads in flight per SM
-  k_pm_interp_tile<R><<<(unsigned)tiles, 128, sm, c->stream>>>(B.cell_start, c->cap, B.u, (const R*)B.phi, M,
-                                                               inv12dx, (R*)B.g);
+  const int sh9 = 3 * (c->cell_depth - c->logM + 3);
+  if (sizeof(R) == 4 && tile_mesh(c)) {
+    const size_t sm = (size_t)13 * (kTy + 5) * (kTy + 8) * sizeof(float);
+    k_pm_interp_tile<float><<<(unsigned)((M / 8) * (M / kTy) * (M / kTy)), kInterpThreads, sm, c->stream>>>(
+        B.cell_start, sh9, c->cap, B.u, (const float*)B.phi, M, (float)inv12dx, (float*)B.g);
+    return;
+  }
+  k_pm_interp_nodes<R><<<(unsigned)((int64_t)M * M * M / 512), 128, (169 * 16 + 3 * 729) * sizeof(R), c->stream>>>(
+      B.cell_start, sh9, c->cap, B.u, (const R*)B.phi, M, inv12dx, (R*)B.g);
 }
 
 // ---- 3D power spectrum of the mesh (forward spectrum of the CIC delta)
@@ -607,7 +776,7 @@ void pk_impl(dzs_ctx* c, int nbins, double* d_part, double* d_out, double shot) 
 // [nbins][3]; d_part is scratch of M * nbins * 3 doubles.  The state must be
 // Morton-sorted with valid keys.
 void launch_pk(dzs_ctx* c, int nbins, double* d_part, double* d_out, double shot) {
-  c->launches += c->mesh_pow2 ? 9 : 22;
+  c->launches += c->mesh_pow2 ? 8 : 16;
   if (c->fp64)
     pk_impl<double>(c, nbins, d_part, d_out, shot);
   else
@@ -631,11 +800,11 @@ void launch_cells(dzs_ctx* c, int depth) {
   k_cell_start<<<grid_for(c->N0 + 1), kThreads, 0, c->stream>>>(c->B.n, c->B.key, sh, ncell, c->B.cell_start);
 }
 
-// depth m = log2 M: the mesh cells of M = 2^m
-void launch_cell_start(dzs_ctx* c) { launch_cells(c, c->logM); }
+// the table the tree and the PM tiles share
+void launch_cell_start(dzs_ctx* c) { launch_cells(c, c->cell_depth); }
 
 void launch_pm_deposit(dzs_ctx* c) {
-  c->launches += c->mesh_pow2 ? 2 : 16;
+  c->launches += !c->mesh_pow2 ? 9 : tile_mesh(c) ? 1 : 2;
   if (c->fp64)
     pm_deposit<double>(c);
   else

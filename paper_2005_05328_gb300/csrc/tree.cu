@@ -18,7 +18,7 @@
 // scan of the per-tile counts of each depth, then a pass in which each owner
 // writes its nodes.  A node's first child index is the number of depth-(j+1)
 // nodes before its start; the child count is the difference to the next node
-// of the same depth.  Node boundaries: down to the PM mesh depth m the cell
+// of the same depth.  Node boundaries: down to the cell table's depth m the cell
 // ends come from the CSR table of the depth-m Morton cells; deeper, a binary
 // search of the keys inside the parent's range.  The numbering depends only
 // on the keys (no atomics), so the tree is deterministic.
@@ -357,7 +357,7 @@ __global__ void k_tree_sums(const int32_t* __restrict__ lvl, int64_t cap, const 
 void launch_tree(dzs_ctx* c) {
   c->launches += 6;
   Buffers& B = c->B;
-  // the depth-m Morton cell table (also the PM deposit's)
+  // the Morton cell table (also the PM tiles')
   launch_cell_start(c);
   const int64_t ntiles = (c->cap + kTreeTile - 1) / kTreeTile;
   int32_t* info = B.group_head;       // [cap] per-particle L, J, g
@@ -368,7 +368,7 @@ void launch_tree(dzs_ctx* c) {
   k_tree_scan<<<kCols, 1024, 0, c->stream>>>(tcount, ntiles, B.lvl_count);
   k_tree_totals<<<1, 32, 0, c->stream>>>(B.lvl_count, c->node_cap, B.counters, B.err);
   k_tree_nodes<<<(unsigned)ntiles, kTreeTile, 0, c->stream>>>(B.n, c->cap, B.key, B.u, info, tcount, ntiles,
-                                                              B.lvl_count, B.cell_start, c->logM, c->P.leaf_bucket,
+                                                              B.lvl_count, B.cell_start, c->cell_depth, c->P.leaf_bucket,
                                                               B.nodes, cfirst, B.parent, B.groups);
   k_tree_link<<<grid_for(c->node_cap, kThreads, 8), kThreads, 0, c->stream>>>(B.lvl_count, B.nodes, cfirst,
                                                                                      B.parent);
