@@ -52,6 +52,7 @@ struct MergeParams {
   int filter;                   // 1 when theta_dzs <= 1/sqrt(3) (geometric only)
   int criterion;                // DZS_CRIT_GEOMETRIC / DZS_CRIT_DYNAMICAL
   double rb;                    // R_lat + b_lat (dynamical)
+  uint64_t rbl;                 // the same as an integer
   double scale;                 // L / 2^32
   double gm0;                   // G m0 = 1.5 Omega_m L^3 / (4 pi N0)
   double alpha;                 // alpha of Eq. 2
@@ -289,6 +290,16 @@ __device__ __forceinline__ void block_first(int64_t first, bool deferred, unsign
   }
 }
 
+// A level whose cells cannot qualify for particle i needs no bounds: the COM lies
+// in i's cell, so d_COM <= d_i + sqrt(3) l_j, and while that is at most T_j
+// (dynamical: R_lat + b_lat, and then for every finer level too) the cell does
+// not merge.  FP32, rounded to the safe side: reach(j) overestimates d_COM by
+// less than 2^-20, `most` underestimates the bound.
+__device__ __forceinline__ bool cannot_reach(float di, int j, uint64_t bound) {
+  const float side = __int_as_float((127 + 32 - j) << 23);  // 2^(32 - j)
+  return (di + 1.7320509f * side) * (1.0f + 0x1p-20f) <= (float)bound * (1.0f - 0x1p-20f);
+}
+
 // kPrefix false: the first pass over every particle (geometric criterion with
 // the member filter): candidates whose cells at the levels that can merge hold
 // at most kDirect particles are decided from direct sums, the others deferred.
@@ -318,15 +329,19 @@ __global__ void k_merge_mark(const int32_t* __restrict__ d_n, int64_t cap, const
     int32_t res = 0;
     bool deferred = false;
     bool cand = true;
-    if (mp.filter) cand = dist2_obs(u[i], u[cap + i], u[2 * cap + i]) > mp.rb2;
+    const uint64_t d2i = dist2_obs(u[i], u[cap + i], u[2 * cap + i]);
+    if (mp.filter) cand = d2i > mp.rb2;
     if (cand) {
       uint64_t ki = key[i];
-      // candidate cells start at depth jstart: its bounds by galloping out
-      // from i (the coarser cells only contain it), deeper ones inside the
-      // previous
-      const int j0 = mp.jstart;
+      // from the first level that can qualify: bounds by galloping out from i
+      // (the coarser cells only contain it), deeper ones inside the previous
+      int j0 = mp.jstart;
+      const float di = sqrtf((float)d2i);
+      if (mp.criterion == DZS_CRIT_GEOMETRIC)
+        while (j0 <= kMaxLevel && (mp.thr[j0] == ~0ull || cannot_reach(di, j0, mp.thr[j0]))) ++j0;
       int64_t lo = 0, hi = n;
       for (int j = j0; j <= kMaxLevel; ++j) {
+        if (mp.criterion == DZS_CRIT_DYNAMICAL && cannot_reach(di, j, mp.rbl)) break;
         int sh = 3 * (kMaxLevel - j);
         uint64_t cell = (ki >> sh) << sh;
         int64_t s, e;
@@ -509,6 +524,7 @@ void launch_merge(dzs_ctx* c, uint64_t rlat) {
   mp.filter = (!dyn && c->P.theta_dzs <= 0.5773502691896257) ? 1 : 0;
   mp.criterion = c->P.dzs_criterion;
   mp.rb = (double)rb;
+  mp.rbl = rb;
   mp.scale = c->scale;
   mp.gm0 = c->gm0;
   mp.alpha = c->P.alpha_dyn;
