@@ -152,7 +152,7 @@ struct Buffers {
   // (list entries x group particles), 5 in-range pairs (0 < r < r_cut),
   // 6 walk work counter, 7 deepest walk stack, 8..11 diagnostics integer sums,
   // 12 walk node tests, 13 walk rounds, 14 a_min^2, 15 scratch, 16 walk units,
-  // 18 crossings of the next step (ring check)
+  // 18 crossings of the next step (ring check), 19 record blocks done
   uint64_t* counters = nullptr;
   double* diag = nullptr;        // [8 + blocks] diagnostics partials
   void* convert = nullptr;       // double [3][cap] conversion scratch
