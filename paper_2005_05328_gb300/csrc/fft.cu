@@ -75,7 +75,7 @@ __device__ __forceinline__ void reg_fft3(cplx<R> (&a)[K], bool inv) {
       w1.y = -w1.y;
       w2.y = -w2.y;
     }
-    const cplx<R> x0 = s0[k], x1 = cmul(s1[k], w1), x2 = cmul(s2[k], w2);
+    const cplx<R> x0 = s0[k], x1 = k ? cmul(s1[k], w1) : s1[k], x2 = k ? cmul(s2[k], w2) : s2[k];
     const cplx<R> t1 = {x1.x + x2.x, x1.y + x2.y}, t2 = {x1.x - x2.x, x1.y - x2.y};
     const cplx<R> m = {x0.x + c * t1.x, x0.y + c * t1.y};
     a[k] = {x0.x + t1.x, x0.y + t1.y};
@@ -109,9 +109,12 @@ __device__ __forceinline__ void reg_fft(cplx<R> (&a)[K], bool inv) {
     for (int b = 0; b < K / 2; ++b) {
       const int j = b & (half - 1);
       const int i0 = ((b >> s) << (s + 1)) + j, i1 = i0 + half;
-      cplx<R> w = tw32(j * (32 / (2 * half)), R(0));
-      if (inv) w.y = -w.y;
-      cplx<R> x = a[i0], y = cmul(a[i1], w);
+      cplx<R> x = a[i0], y = a[i1];
+      if (j != 0) {  // (j = 0: the factor is 1)
+        cplx<R> w = tw32(j * (32 / (2 * half)), R(0));
+        if (inv) w.y = -w.y;
+        y = cmul(y, w);
+      }
       a[i0] = {x.x + y.x, x.y + y.y};
       a[i1] = {x.x - y.x, x.y - y.y};
     }
@@ -157,7 +160,7 @@ __device__ __forceinline__ void stepA_smem(cplx<R>* buf, int W, int col, int j2,
   for (int j1 = 0; j1 < N1; ++j1) a[j1] = buf[sidx((j1 * N2 + j2), col, W)];
   reg_fft<R, N1>(a, inv);
 #pragma unroll
-  for (int k1 = 0; k1 < N1; ++k1) a[k1] = cmul(a[k1], twn(tw, j2 * k1, N, inv));
+  for (int k1 = 1; k1 < N1; ++k1) a[k1] = cmul(a[k1], twn(tw, j2 * k1, N, inv));
 #pragma unroll
   for (int k1 = 0; k1 < N1; ++k1) buf[sidx((k1 * N2 + j2), col, W)] = a[k1];
 }
@@ -285,7 +288,8 @@ __global__ void k_fft_cols(cplx<R>* __restrict__ spec, int W, int axis, int mode
     for (int j1 = 0; j1 < N1; ++j1) a[j1] = valid ? spec[base + (j1 * N2 + r) * es + kz0 + col] : cplx<R>{0, 0};
     reg_fft<R, N1>(a, inv);
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) buf[sidx((k1 * N2 + r), col, W)] = cmul(a[k1], twn(tw, r * k1, N, inv));
+    for (int k1 = 0; k1 < N1; ++k1)
+      buf[sidx((k1 * N2 + r), col, W)] = k1 ? cmul(a[k1], twn(tw, r * k1, N, inv)) : a[k1];
   }
   __syncthreads();
   cplx<R> b[N2];
@@ -322,7 +326,8 @@ __global__ void k_fft_cols(cplx<R>* __restrict__ spec, int W, int axis, int mode
   if (r < N1) {
     reg_fft<R, N2>(b, true);
 #pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) buf[sidx((k2 * N1 + r), col, W)] = cmul(b[k2], twn(tw, r * k2, N, true));
+    for (int k2 = 0; k2 < N2; ++k2)
+      buf[sidx((k2 * N1 + r), col, W)] = k2 ? cmul(b[k2], twn(tw, r * k2, N, true)) : b[k2];
   }
   __syncthreads();
   if (r < N2) {
@@ -579,6 +584,18 @@ int cols_per_block() {
   return w;
 }
 
+// columns of a Y or X block: the n/2 + 1 columns of a line split evenly over the
+// fewest blocks (the one column beyond a power of two would leave a whole block
+// transforming zeros: mesh 64, 33 columns, 17 + 16 instead of 32 + 1)
+template <class R, int N>
+int cols_balanced() {
+  constexpr int HN = N / 2 + 1;
+  int w = cols_per_block<R, N>();
+  const int blocks = (HN + w - 1) / w;
+  const int even = (HN + blocks - 1) / blocks;
+  return (size_t)srows(even) * N * sizeof(cplx<R>) <= 48 * 1024 ? even : w;
+}
+
 template <class R, int N>
 void launch_r2c_zy(dzs_ctx* c, const R* in, cplx<R>* out, const cplx<R>* tw, bool do_x) {
   if constexpr (three_factor<R>(N)) {
@@ -590,9 +607,10 @@ void launch_r2c_zy(dzs_ctx* c, const R* in, cplx<R>* out, const cplx<R>* tw, boo
     const size_t sm = (size_t)N * srows(W) * sizeof(cplx<R>);
     const int64_t npairs = (int64_t)N * N / 2;
     k_fft_z_r2c<R, N><<<(unsigned)((npairs + W - 1) / W), threads, sm, c->stream>>>(in, out, W, npairs, tw);
-    const int ncb = (N / 2 + 1 + W - 1) / W;
-    k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(out, W, 1, 0, tw, nullptr, (R)0);
-    if (do_x) k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(out, W, 0, 0, tw, nullptr, (R)0);
+    const int Wc = cols_balanced<R, N>(), ncb = (N / 2 + 1 + Wc - 1) / Wc, cthreads = Wc * Split<N>::N1;
+    const size_t csm = (size_t)N * srows(Wc) * sizeof(cplx<R>);
+    k_fft_cols<R, N><<<N * ncb, cthreads, csm, c->stream>>>(out, Wc, 1, 0, tw, nullptr, (R)0);
+    if (do_x) k_fft_cols<R, N><<<N * ncb, cthreads, csm, c->stream>>>(out, Wc, 0, 0, tw, nullptr, (R)0);
   }
 }
 
@@ -606,9 +624,10 @@ void launch_c2r(dzs_ctx* c, cplx<R>* in, R* out, const cplx<R>* tw, const R* gre
     const int threads = W * Split<N>::N1;
     const size_t sm = (size_t)N * srows(W) * sizeof(cplx<R>);
     const int64_t npairs = (int64_t)N * N / 2;
-    const int ncb = (N / 2 + 1 + W - 1) / W;
-    k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(in, W, 0, green ? 2 : 1, tw, green, gfac);
-    k_fft_cols<R, N><<<N * ncb, threads, sm, c->stream>>>(in, W, 1, 1, tw, nullptr, (R)0);
+    const int Wc = cols_balanced<R, N>(), ncb = (N / 2 + 1 + Wc - 1) / Wc, cthreads = Wc * Split<N>::N1;
+    const size_t csm = (size_t)N * srows(Wc) * sizeof(cplx<R>);
+    k_fft_cols<R, N><<<N * ncb, cthreads, csm, c->stream>>>(in, Wc, 0, green ? 2 : 1, tw, green, gfac);
+    k_fft_cols<R, N><<<N * ncb, cthreads, csm, c->stream>>>(in, Wc, 1, 1, tw, nullptr, (R)0);
     k_fft_z_c2r<R, N><<<(unsigned)((npairs + W - 1) / W), threads, sm, c->stream>>>(in, out, W, npairs, tw);
   }
 }
