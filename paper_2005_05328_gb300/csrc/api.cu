@@ -155,6 +155,17 @@ struct Plan {
     if (e_ != cudaSuccess) return fail(c, DZS_ECUDA, #call, cudaGetErrorString(e_)); \
   } while (0)
 
+// the same amid copies queued on the stream: they end before the caller's buffer
+// may go
+#define CKQ(call)                                                                  \
+  do {                                                                             \
+    cudaError_t e_ = (call);                                                       \
+    if (e_ != cudaSuccess) {                                                       \
+      cudaStreamSynchronize(c->stream);                                            \
+      return fail(c, DZS_ECUDA, #call, cudaGetErrorString(e_));                    \
+    }                                                                              \
+  } while (0)
+
 // host-side allocation-failure injection (tests): the k-th device
 // allocation from now on fails as if the device were out of memory
 std::atomic<int> g_fail_alloc{0};
@@ -195,13 +206,28 @@ dzs_status device_error_status(dzs_ctx* c, uint32_t err) {
   return DZS_OK;
 }
 
-dzs_status check_device_errors(dzs_ctx* c) {
+// particle count, error word and counters lie side by side in the arena
+// (Plan): one copy reads all three
+struct DeviceStatus {
+  int32_t n;
+  uint8_t pad0[252];
+  uint32_t err;
+  uint8_t pad1[252];
+  uint64_t counters[32];
+};
+static_assert(sizeof(DeviceStatus) == 768, "three 256-byte arena blocks");
+
+// waits for the stream; DZS_EDEVICE on a failure, else the error word's status
+dzs_status read_status(dzs_ctx* c, DeviceStatus* st) {
   cudaError_t e = cudaStreamSynchronize(c->stream);
+  if (e == cudaSuccess) e = cudaMemcpy(st, c->B.n, sizeof *st, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return fail(c, DZS_EDEVICE, "device failure", cudaGetErrorString(e));
-  uint32_t err = 0;
-  e = cudaMemcpy(&err, c->B.err, sizeof(uint32_t), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return fail(c, DZS_EDEVICE, "device failure", cudaGetErrorString(e));
-  return device_error_status(c, err);
+  return device_error_status(c, st->err);
+}
+
+dzs_status check_device_errors(dzs_ctx* c) {
+  DeviceStatus st;
+  return read_status(c, &st);
 }
 
 dzs_status guard(dzs_ctx* c) {
@@ -658,10 +684,10 @@ dzs_status dzs_lightcone_drain(dzs_ctx* c, dzs_lc_record* host_buf, size_t cap, 
   if (s) return s;
   if (n_out) *n_out = 0;
   if (!host_buf && cap) return fail(c, DZS_EINVAL, "host_buf is NULL");
-  s = check_device_errors(c);
+  DeviceStatus st;
+  s = read_status(c, &st);
   if (s) return s;
-  uint64_t ctr[2];
-  CK(cudaMemcpy(ctr, c->B.counters, sizeof ctr, cudaMemcpyDeviceToHost));
+  const uint64_t* ctr = st.counters;
   uint64_t avail = ctr[0] - c->drained;
   uint64_t take = avail < cap ? avail : cap;
   uint64_t done = 0;
@@ -759,11 +785,10 @@ dzs_status dzs_lightcone_drain_step(dzs_ctx* c, int32_t step, dzs_lc_record* hos
 dzs_status dzs_get_count(dzs_ctx* c, size_t* n, int32_t* step) {
   dzs_status s = guard(c);
   if (s) return s;
-  s = check_device_errors(c);
+  DeviceStatus st;
+  s = read_status(c, &st);
   if (s) return s;
-  int32_t hn = 0;
-  CK(cudaMemcpy(&hn, c->B.n, sizeof hn, cudaMemcpyDeviceToHost));
-  if (n) *n = (size_t)hn;
+  if (n) *n = (size_t)st.n;
   if (step) *step = c->step;
   return DZS_OK;
 }
@@ -916,23 +941,25 @@ bool same_physics(const dzs_params& a, const dzs_params& b) {
 }  // namespace
 
 dzs_status dzs_checkpoint_bytes(dzs_ctx* c, size_t* bytes) {
-  size_t n = 0;
-  dzs_status s = dzs_get_count(c, &n, nullptr);
+  dzs_status s = guard(c);
+  if (s) return s;
+  DeviceStatus st;
+  s = read_status(c, &st);
   if (s) return s;
   if (!bytes) return fail(c, DZS_EINVAL, "bytes is NULL");
-  uint64_t head = 0;
-  CK(cudaMemcpy(&head, c->B.counters, sizeof head, cudaMemcpyDeviceToHost));
-  *bytes = ckpt_size(c, n, head - c->drained);
+  *bytes = ckpt_size(c, (uint64_t)st.n, st.counters[0] - c->drained);
   return DZS_OK;
 }
 
 dzs_status dzs_checkpoint(dzs_ctx* c, void* host_buf, size_t cap, size_t* written) {
-  size_t n = 0;
-  dzs_status s = dzs_get_count(c, &n, nullptr);
+  dzs_status s = guard(c);
   if (s) return s;
+  DeviceStatus st;
+  s = read_status(c, &st);
+  if (s) return s;
+  const size_t n = (size_t)st.n;
   if (!c->have_state) return fail(c, DZS_ESTATE, "no particle state");
-  uint64_t ctr[2];
-  CK(cudaMemcpy(ctr, c->B.counters, sizeof ctr, cudaMemcpyDeviceToHost));
+  const uint64_t* ctr = st.counters;
   const uint64_t pending = ctr[0] - c->drained;
   const size_t need = ckpt_size(c, n, pending), rsz = c->fp64 ? 8 : 4;
   if (written) *written = 0;
@@ -948,26 +975,29 @@ dzs_status dzs_checkpoint(dzs_ctx* c, void* host_buf, size_t cap, size_t* writte
   h.pending = pending;
   h.dropped = ctr[1];
   h.rsz = rsz;
+  // all copies queued on the stream, one wait: each waiting on its own cost ~8 us
   memcpy(o, &h, sizeof h);
   o += sizeof h;
-  for (int ax = 0; ax < 3; ++ax, o += 4 * n) CK(cudaMemcpy(o, c->B.u + ax * c->cap, 4 * n, cudaMemcpyDeviceToHost));
+  for (int ax = 0; ax < 3; ++ax, o += 4 * n)
+    CKQ(cudaMemcpyAsync(o, c->B.u + ax * c->cap, 4 * n, cudaMemcpyDeviceToHost, c->stream));
   for (int ax = 0; ax < 3; ++ax, o += rsz * n)
-    CK(cudaMemcpy(o, (char*)c->B.p + ax * c->cap * rsz, rsz * n, cudaMemcpyDeviceToHost));
+    CKQ(cudaMemcpyAsync(o, (char*)c->B.p + ax * c->cap * rsz, rsz * n, cudaMemcpyDeviceToHost, c->stream));
   for (int ax = 0; ax < 3; ++ax, o += rsz * n)
-    CK(cudaMemcpy(o, (char*)c->B.g + ax * c->cap * rsz, rsz * n, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(o, c->B.k, 4 * n, cudaMemcpyDeviceToHost));
+    CKQ(cudaMemcpyAsync(o, (char*)c->B.g + ax * c->cap * rsz, rsz * n, cudaMemcpyDeviceToHost, c->stream));
+  CKQ(cudaMemcpyAsync(o, c->B.k, 4 * n, cudaMemcpyDeviceToHost, c->stream));
   o += 4 * n;
-  CK(cudaMemcpy(o, c->B.id, 4 * n, cudaMemcpyDeviceToHost));
+  CKQ(cudaMemcpyAsync(o, c->B.id, 4 * n, cudaMemcpyDeviceToHost, c->stream));
   o += 4 * n;
-  CK(cudaMemcpy(o, c->B.fl, n, cudaMemcpyDeviceToHost));
+  CKQ(cudaMemcpyAsync(o, c->B.fl, n, cudaMemcpyDeviceToHost, c->stream));
   o += n;
   for (uint64_t done = 0; done < pending;) {
     uint64_t slot = (c->drained + done) % c->ring_cap, chunk = c->ring_cap - slot;
     if (chunk > pending - done) chunk = pending - done;
-    CK(cudaMemcpy(o, c->B.ring + slot, chunk * sizeof(dzs_lc_record), cudaMemcpyDeviceToHost));
+    CKQ(cudaMemcpyAsync(o, c->B.ring + slot, chunk * sizeof(dzs_lc_record), cudaMemcpyDeviceToHost, c->stream));
     o += chunk * sizeof(dzs_lc_record);
     done += chunk;
   }
+  CK(cudaStreamSynchronize(c->stream));
   if (written) *written = need;
   return DZS_OK;
 }
@@ -984,26 +1014,29 @@ dzs_status dzs_restore(dzs_ctx* c, const void* host_buf, size_t len) {
   if (h.n > (uint64_t)c->cap || h.step > (uint64_t)c->P.nsteps || h.pending > c->ring_cap ||
       h.bytes != ckpt_size(c, h.n, h.pending) || len < h.bytes)
     return fail(c, DZS_EINVAL, "inconsistent checkpoint");
-  CK(cudaStreamSynchronize(c->stream));
+  // everything queued on the stream behind the work in flight, one wait at the
+  // end (the caller's buffer and the locals below are read until then)
   const size_t n = h.n;
   const char* o = (const char*)host_buf + sizeof h;
-  for (int ax = 0; ax < 3; ++ax, o += 4 * n) CK(cudaMemcpy(c->B.u + ax * c->cap, o, 4 * n, cudaMemcpyHostToDevice));
+  for (int ax = 0; ax < 3; ++ax, o += 4 * n)
+    CKQ(cudaMemcpyAsync(c->B.u + ax * c->cap, o, 4 * n, cudaMemcpyHostToDevice, c->stream));
   for (int ax = 0; ax < 3; ++ax, o += rsz * n)
-    CK(cudaMemcpy((char*)c->B.p + ax * c->cap * rsz, o, rsz * n, cudaMemcpyHostToDevice));
+    CKQ(cudaMemcpyAsync((char*)c->B.p + ax * c->cap * rsz, o, rsz * n, cudaMemcpyHostToDevice, c->stream));
   for (int ax = 0; ax < 3; ++ax, o += rsz * n)
-    CK(cudaMemcpy((char*)c->B.g + ax * c->cap * rsz, o, rsz * n, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(c->B.k, o, 4 * n, cudaMemcpyHostToDevice));
+    CKQ(cudaMemcpyAsync((char*)c->B.g + ax * c->cap * rsz, o, rsz * n, cudaMemcpyHostToDevice, c->stream));
+  CKQ(cudaMemcpyAsync(c->B.k, o, 4 * n, cudaMemcpyHostToDevice, c->stream));
   o += 4 * n;
-  CK(cudaMemcpy(c->B.id, o, 4 * n, cudaMemcpyHostToDevice));
+  CKQ(cudaMemcpyAsync(c->B.id, o, 4 * n, cudaMemcpyHostToDevice, c->stream));
   o += 4 * n;
-  CK(cudaMemcpy(c->B.fl, o, n, cudaMemcpyHostToDevice));
+  CKQ(cudaMemcpyAsync(c->B.fl, o, n, cudaMemcpyHostToDevice, c->stream));
   o += n;
-  if (h.pending) CK(cudaMemcpy(c->B.ring, o, h.pending * sizeof(dzs_lc_record), cudaMemcpyHostToDevice));
+  if (h.pending) CKQ(cudaMemcpyAsync(c->B.ring, o, h.pending * sizeof(dzs_lc_record), cudaMemcpyHostToDevice, c->stream));
   uint64_t ctr[2] = {h.pending, h.dropped};
-  CK(cudaMemcpy(c->B.counters, ctr, sizeof ctr, cudaMemcpyHostToDevice));
+  CKQ(cudaMemcpyAsync(c->B.counters, ctr, sizeof ctr, cudaMemcpyHostToDevice, c->stream));
   int32_t nn = (int32_t)n;
-  CK(cudaMemcpy(c->B.n, &nn, sizeof nn, cudaMemcpyHostToDevice));
-  CK(cudaMemset(c->B.err, 0, 16));
+  CKQ(cudaMemcpyAsync(c->B.n, &nn, sizeof nn, cudaMemcpyHostToDevice, c->stream));
+  CKQ(cudaMemsetAsync(c->B.err, 0, 16, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
   c->drained = 0;
   c->step = (int32_t)h.step;
   c->have_state = true;
