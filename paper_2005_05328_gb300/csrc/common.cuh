@@ -151,7 +151,7 @@ struct Buffers {
   // [32]: 0 ring head, 1 records dropped, 2 groups, 3 nodes, 4 listed pairs
   // (list entries x group particles), 5 in-range pairs (0 < r < r_cut),
   // 6 walk work counter, 7 deepest walk stack, 8..11 diagnostics integer sums,
-  // 12 walk node tests, 13 walk rounds, 14 a_min^2, 15 scratch, 16 walk units,
+  // 12 walk node tests, 13 walk rounds, 14 a_min^2, 15 scratch, 16 tree blocks done, 17 merge blocks done,
   // 18 crossings of the next step (ring check), 19 record blocks done
   uint64_t* counters = nullptr;
   double* diag = nullptr;        // [8 + blocks] diagnostics partials

@@ -34,6 +34,7 @@
 // that changes, into the spare arrays, and copies that tail back: a step that
 // merges nothing writes nothing.
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -261,33 +262,54 @@ __device__ __forceinline__ int64_t gallop_up(const uint64_t* __restrict__ key, i
   return lower_bound_key(key, lo, hi, x);
 }
 
-// smallest index with a nonzero mark in this block, and whether any candidate
-// was deferred: one atomic each per block
-__device__ __forceinline__ void block_first(int64_t first, bool deferred, unsigned long long* __restrict__ first_slot,
-                                            unsigned* __restrict__ need) {
-  __shared__ unsigned long long wmin[32];
+// particles of one block of the mark and write kernels: consecutive, so that
+// the blocks' survivor counts give every survivor its place
+__device__ __forceinline__ int64_t block_share(int64_t n) {
+  return ((n + gridDim.x - 1) / gridDim.x + kThreads - 1) / kThreads * kThreads;
+}
+
+// this block's survivors to kept[block]; the smallest index with a nonzero mark
+// (as its complement: 0 when there is none) and whether any candidate was
+// deferred, one atomic each per block
+__device__ __forceinline__ void block_result(int64_t first, bool deferred, unsigned kept,
+                                             int32_t* __restrict__ block_kept,
+                                             unsigned long long* __restrict__ first_slot, unsigned* __restrict__ need) {
+  __shared__ unsigned long long wmax[32];
   __shared__ int wdef[32];
-  unsigned long long f = (unsigned long long)first;
+  __shared__ unsigned wkept[32];
+  unsigned long long f = ~(unsigned long long)first;  // none: INT64_MAX, the smallest complement
+  if (first == INT64_MAX) f = 0;
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long t = __shfl_down_sync(0xffffffffu, f, o);
-    f = t < f ? t : f;
+    f = t > f ? t : f;
+    kept += __shfl_down_sync(0xffffffffu, kept, o);
   }
   const int d = __any_sync(0xffffffffu, deferred) ? 1 : 0;
   if ((threadIdx.x & 31) == 0) {
-    wmin[threadIdx.x >> 5] = f;
+    wmax[threadIdx.x >> 5] = f;
     wdef[threadIdx.x >> 5] = d;
+    wkept[threadIdx.x >> 5] = kept;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned long long m = ~0ull;
+    unsigned long long m = 0;
     int any = 0;
+    unsigned sum = 0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      m = wmin[w] < m ? wmin[w] : m;
+      m = wmax[w] > m ? wmax[w] : m;
       any |= wdef[w];
+      sum += wkept[w];
     }
-    if (m != ~0ull) atomicMin(first_slot, m);
-    if (any) atomicOr(need, 1u);
+    block_kept[blockIdx.x] = (int32_t)sum;
+    if (m) atomicMax(first_slot, m);
+    if (any && need) atomicOr(need, 1u);
   }
+}
+
+// first changed particle, n when there is none
+__device__ __forceinline__ int64_t first_of(const unsigned long long* __restrict__ slot, int64_t n) {
+  const unsigned long long f = *slot;
+  return f && (int64_t)~f < n ? (int64_t)~f : n;
 }
 
 // A level whose cells cannot qualify for particle i needs no bounds: the COM lies
@@ -310,9 +332,9 @@ template <bool kPrefix>
 __global__ void k_merge_mark(const int32_t* __restrict__ d_n, int64_t cap, const uint64_t* __restrict__ key,
                              const uint32_t* __restrict__ u, const uint32_t* __restrict__ kk,
                              const uint64_t* __restrict__ pre, int32_t* __restrict__ mend,
-                             int32_t* __restrict__ keep, MergeParams mp, unsigned long long* __restrict__ first_slot,
-                             unsigned* __restrict__ need) {
-  if (kPrefix && !*need) return;
+                             int32_t* __restrict__ block_kept, MergeParams mp,
+                             unsigned long long* __restrict__ first_slot, unsigned* __restrict__ need) {
+  if (kPrefix && need && !*need) return;
   const int64_t n = *d_n;
   const uint64_t* PK = pre;
   const uint64_t* PS = pre + (cap + 1);
@@ -324,8 +346,16 @@ __global__ void k_merge_mark(const int32_t* __restrict__ d_n, int64_t cap, const
   }
   int64_t first = INT64_MAX;
   bool deferred_any = false;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (kPrefix && mp.filter && mend[i] != kDeferred) continue;
+  unsigned kept = 0;
+  const int64_t share = block_share(n), b0 = blockIdx.x * share, b1 = b0 + share < n ? b0 + share : n;
+  for (int64_t i = b0 + threadIdx.x; i < b1; i += kThreads) {
+    if (kPrefix && mp.filter) {
+      const int32_t m = mend[i];
+      if (m != kDeferred) {
+        kept += m >= 0 ? 1u : 0u;
+        continue;
+      }
+    }
     int32_t res = 0;
     bool deferred = false;
     bool cand = true;
@@ -392,31 +422,55 @@ __global__ void k_merge_mark(const int32_t* __restrict__ d_n, int64_t cap, const
       }
     }
     mend[i] = deferred ? kDeferred : res;
-    keep[i] = res >= 0 ? 1 : 0;
+    kept += !deferred && res >= 0 ? 1u : 0u;
     if (res != 0 && i < first) first = i;
     deferred_any = deferred_any || deferred;
   }
-  block_first(first, deferred_any, first_slot, need);
+  block_result(first, deferred_any, kept, block_kept, first_slot, need);
 }
 
 // the compacted state from the first changed particle on, into the spare
-// arrays (rank = exclusive scan of keep); merged cells summed directly
+// arrays (place = survivors of the blocks before, then in the block); merged
+// cells summed directly; *d_n_out = survivors
 template <class R>
-__global__ void k_merge_write(const int32_t* __restrict__ d_n, int64_t cap, const int32_t* __restrict__ mend,
-                              const int32_t* __restrict__ rank, const uint64_t* __restrict__ key,
+__global__ void __launch_bounds__(kThreads)
+    k_merge_write(const int32_t* __restrict__ d_n, int64_t cap, const int32_t* __restrict__ mend,
+                              const int32_t* __restrict__ block_kept, const uint64_t* __restrict__ key,
                               const uint32_t* __restrict__ u, const R* __restrict__ p,
                               const uint32_t* __restrict__ k, const uint32_t* __restrict__ id,
                               const uint8_t* __restrict__ fl, const unsigned long long* __restrict__ first_slot,
                               uint64_t* __restrict__ key2, uint32_t* __restrict__ u2, R* __restrict__ p2,
                               uint32_t* __restrict__ k2, uint32_t* __restrict__ id2, uint8_t* __restrict__ fl2,
                               int32_t* __restrict__ d_n_out) {
+  __shared__ unsigned wsum[kThreads / 32];
   const int64_t n = *d_n;
-  const int64_t first = *first_slot < (unsigned long long)n ? (int64_t)*first_slot : n;
-  for (int64_t i = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int32_t m = mend[i];
-    if (m < 0) continue;
-    int64_t j = rank[i];
+  const int64_t first = first_of(first_slot, n);
+  const int64_t share = block_share(n), b0 = blockIdx.x * share, b1 = b0 + share < n ? b0 + share : n;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool last = blockIdx.x == gridDim.x - 1;
+  if (b1 <= first && !last) return;  // nothing of this block changes
+  unsigned before = 0;
+  for (int q = threadIdx.x; q < (int)blockIdx.x; q += kThreads) before += (unsigned)block_kept[q];
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_down_sync(0xffffffffu, before, o);
+  if (lane == 0) wsum[w] = before;
+  __syncthreads();
+  before = 0;
+  for (int q = 0; q < kThreads / 32; ++q) before += wsum[q];
+  if (last && threadIdx.x == 0) *d_n_out = (int32_t)before + block_kept[blockIdx.x];
+  if (b1 <= first) return;
+  for (int64_t i0 = b0; i0 < b1; i0 += kThreads) {
+    const int64_t i = i0 + threadIdx.x;
+    const int32_t m = i < b1 ? mend[i] : -1;
+    const unsigned bal = __ballot_sync(0xffffffffu, m >= 0);
+    __syncthreads();
+    if (lane == 0) wsum[w] = __popc(bal);
+    __syncthreads();
+    int64_t j = before + __popc(bal & ((1u << lane) - 1u));
+    for (int q = 0; q < kThreads / 32; ++q) {
+      if (q < w) j += wsum[q];
+      before += wsum[q];
+    }
+    if (m < 0 || i < first) continue;
     if (m == 0) {
       for (int ax = 0; ax < 3; ++ax) {
         u2[ax * cap + j] = u[ax * cap + i];
@@ -450,20 +504,21 @@ __global__ void k_merge_write(const int32_t* __restrict__ d_n, int64_t cap, cons
     id2[j] = idm;
     fl2[j] = (uint8_t)(kFlMerged | kFlCrossed);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *d_n_out = rank[n];
 }
 
-// the changed tail [first, n_new) back into the state arrays
+// the changed tail [first, n_new) back into the state arrays; the block that
+// finishes last (all have read the slots) sets the count and clears the slots
+// for the next merge
 template <class R>
-__global__ void k_merge_copyback(const int32_t* __restrict__ d_n_new, int64_t cap,
-                                 const unsigned long long* __restrict__ first_slot, const uint64_t* __restrict__ key2,
+__global__ void k_merge_copyback(int32_t* d_n, int64_t cap, unsigned long long* first_slot, unsigned* need,
+                                 unsigned* done, const uint64_t* __restrict__ key2,
                                  const uint32_t* __restrict__ u2, const R* __restrict__ p2,
                                  const uint32_t* __restrict__ k2, const uint32_t* __restrict__ id2,
                                  const uint8_t* __restrict__ fl2, uint64_t* __restrict__ key, uint32_t* __restrict__ u,
                                  R* __restrict__ p, uint32_t* __restrict__ k, uint32_t* __restrict__ id,
                                  uint8_t* __restrict__ fl) {
-  const int64_t n = *d_n_new;
-  const int64_t first = *first_slot < (unsigned long long)n ? (int64_t)*first_slot : n;
+  const int64_t n = d_n[1];
+  const int64_t first = first_of(first_slot, n);
   for (int64_t i = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     for (int ax = 0; ax < 3; ++ax) {
@@ -474,6 +529,16 @@ __global__ void k_merge_copyback(const int32_t* __restrict__ d_n_new, int64_t ca
     k[i] = k2[i];
     id[i] = id2[i];
     fl[i] = fl2[i];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(done, 1u) == gridDim.x - 1) {
+      d_n[0] = (int32_t)n;
+      *first_slot = 0;
+      *need = 0;
+      *done = 0;
+    }
   }
 }
 
@@ -534,48 +599,37 @@ void launch_merge(dzs_ctx* c, uint64_t rlat) {
   }
   uint64_t* slot = c->B.counters + 14;
   mp.amin2_slot = slot;
+  // zero between merges (the last block of the copy-back clears them)
   unsigned long long* first = (unsigned long long*)(c->B.counters + 22);
   unsigned* need = (unsigned*)(c->B.counters + 23);
-  cudaMemsetAsync(first, 0xff, sizeof(uint64_t), c->stream);
+  unsigned* done = (unsigned*)(c->B.counters + 17);
   int nchunks = (int)((c->cap + kChunk) / kChunk);
   uint64_t* tot = (uint64_t*)B.blocksum;
-  int32_t* keep = B.iscan + (c->cap + 1);
-  int32_t* rank = B.iscan;
-  int grid = grid_for(c->N0);
-  if (mp.filter) {
-    c->launches += 1;
-    cudaMemsetAsync(need, 0, sizeof(unsigned), c->stream);
-    k_merge_mark<false><<<grid, kThreads, 0, c->stream>>>(B.n, c->cap, B.key, B.u, B.k, B.prefix, B.mend, keep, mp,
+  int32_t* kept = B.iscan;  // survivors of each block
+  const int grid = grid_for(c->cap);
+  c->launches += mp.filter ? 7 : 6;
+  if (mp.filter)
+    k_merge_mark<false><<<grid, kThreads, 0, c->stream>>>(B.n, c->cap, B.key, B.u, B.k, B.prefix, B.mend, kept, mp,
                                                           first, need);
-  } else {
-    cudaMemsetAsync(need, 1, sizeof(unsigned), c->stream);  // nonzero: every particle takes the prefix pass
-  }
   // prefix sums and the second mark pass: they return at once unless needed
-  c->launches += 4;
-  k_prefix_totals<<<nchunks, 256, 0, c->stream>>>(B.n, c->cap, B.u, B.k, tot, need);
-  k_prefix_scan_totals<<<4, 1024, 0, c->stream>>>(tot, nchunks, need);
-  k_prefix_apply<<<nchunks, 256, 0, c->stream>>>(B.n, c->cap, B.u, B.k, tot, nchunks, B.prefix, need);
-  k_merge_mark<true><<<grid, kThreads, 0, c->stream>>>(B.n, c->cap, B.key, B.u, B.k, B.prefix, B.mend, keep, mp,
-                                                       first, need);
-  c->launches += 5;
-  exclusive_scan_i32(c, keep, rank, B.n, c->cap);
-  if (c->fp64) {
-    k_merge_write<double><<<grid, kThreads, 0, c->stream>>>(
-        B.n, c->cap, B.mend, rank, B.key, B.u, (const double*)B.p, B.k, B.id, B.fl, first, B.key2, B.u2,
-        (double*)B.p2, B.k2, B.id2, B.fl2, B.n + 1);
-    k_merge_copyback<double><<<grid, kThreads, 0, c->stream>>>(B.n + 1, c->cap, first, B.key2, B.u2,
-                                                               (const double*)B.p2, B.k2, B.id2, B.fl2, B.key, B.u,
-                                                               (double*)B.p, B.k, B.id, B.fl);
-  } else {
-    k_merge_write<float><<<grid, kThreads, 0, c->stream>>>(
-        B.n, c->cap, B.mend, rank, B.key, B.u, (const float*)B.p, B.k, B.id, B.fl, first, B.key2, B.u2,
-        (float*)B.p2, B.k2, B.id2, B.fl2, B.n + 1);
-    k_merge_copyback<float><<<grid, kThreads, 0, c->stream>>>(B.n + 1, c->cap, first, B.key2, B.u2,
-                                                              (const float*)B.p2, B.k2, B.id2, B.fl2, B.key, B.u,
-                                                              (float*)B.p, B.k, B.id, B.fl);
-  }
-  // new count staged in n[1] (every thread of the write kernel read n[0])
-  cudaMemcpyAsync(B.n, B.n + 1, sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream);
+  // (without the filter every particle takes them)
+  unsigned* when = mp.filter ? need : nullptr;
+  k_prefix_totals<<<nchunks, 256, 0, c->stream>>>(B.n, c->cap, B.u, B.k, tot, when);
+  k_prefix_scan_totals<<<4, 1024, 0, c->stream>>>(tot, nchunks, when);
+  k_prefix_apply<<<nchunks, 256, 0, c->stream>>>(B.n, c->cap, B.u, B.k, tot, nchunks, B.prefix, when);
+  k_merge_mark<true><<<grid, kThreads, 0, c->stream>>>(B.n, c->cap, B.key, B.u, B.k, B.prefix, B.mend, kept, mp, first,
+                                                       when);
+  auto finish = [&](auto* p, auto* p2) {
+    using R = std::remove_pointer_t<decltype(p)>;
+    k_merge_write<R><<<grid, kThreads, 0, c->stream>>>(B.n, c->cap, B.mend, kept, B.key, B.u, p, B.k, B.id, B.fl, first,
+                                                       B.key2, B.u2, p2, B.k2, B.id2, B.fl2, B.n + 1);
+    k_merge_copyback<R><<<grid, kThreads, 0, c->stream>>>(B.n, c->cap, first, need, done, B.key2, B.u2, p2, B.k2, B.id2,
+                                                          B.fl2, B.key, B.u, p, B.k, B.id, B.fl);
+  };
+  if (c->fp64)
+    finish((double*)B.p, (double*)B.p2);
+  else
+    finish((float*)B.p, (float*)B.p2);
 }
 
 }  // namespace dzs

@@ -114,8 +114,12 @@ __global__ void __launch_bounds__(kTreeTile) k_tree_count(const int32_t* __restr
   }
 }
 
-// block c: exclusive scan of column c of the tile counts, column total to tot[c]
-__global__ void k_tree_scan(int32_t* __restrict__ tcount, int64_t ntiles, int32_t* __restrict__ tot) {
+// block c: exclusive scan of column c of the tile counts, column total to
+// lvl[c].  The block that finishes last turns the totals into the node and group
+// counts (a tree above the node capacity is not built: error bit, zero nodes and
+// groups) and clears what the walk accumulates into.
+__global__ void k_tree_scan(int32_t* __restrict__ tcount, int64_t ntiles, int32_t* lvl, int64_t node_cap,
+                            uint64_t* counters, uint32_t* __restrict__ err) {
   __shared__ int32_t warp_tot[32];
   __shared__ int32_t carry;
   int32_t* col = tcount + (int64_t)blockIdx.x * ntiles;
@@ -148,23 +152,24 @@ __global__ void k_tree_scan(int32_t* __restrict__ tcount, int64_t ntiles, int32_
     if (threadIdx.x == blockDim.x - 1) carry = ex + v;
     __syncthreads();
   }
-  if (threadIdx.x == 0) tot[blockIdx.x] = carry;
-}
-
-// node counts per depth and the group count; a tree above the node capacity
-// is not built (error bit, zero nodes and groups)
-__global__ void k_tree_totals(int32_t* __restrict__ lvl, int64_t node_cap, uint64_t* __restrict__ counters,
-                              uint32_t* __restrict__ err) {
   if (threadIdx.x != 0) return;
+  volatile int32_t* tot = lvl;
+  tot[blockIdx.x] = carry;
+  __threadfence();
+  if (atomicAdd((unsigned*)(counters + 16), 1u) != gridDim.x - 1) return;
+  __threadfence();
   int64_t total = 0;
-  for (int j = 0; j <= kMaxLevel; ++j) total += lvl[j];
+  for (int j = 0; j <= kMaxLevel; ++j) total += tot[j];
   if (total > node_cap) {
     atomicOr(err, kErrNodes);
-    for (int j = 0; j < kCols; ++j) lvl[j] = 0;
+    for (int j = 0; j < kCols; ++j) tot[j] = 0;
     total = 0;
   }
-  counters[2] = (uint64_t)lvl[kCols - 1];
+  counters[2] = (uint64_t)tot[kCols - 1];
   counters[3] = (uint64_t)total;
+  counters[6] = 0;   // the walk's work counter
+  counters[24] = 0;  // its largest spline radius
+  *(unsigned*)(counters + 16) = 0u;  // blocks done, for the next tree
 }
 
 // every owner writes its nodes: index = (nodes of shallower depths) + (nodes of
@@ -355,7 +360,7 @@ __global__ void k_tree_sums(const int32_t* __restrict__ lvl, int64_t cap, const 
 }  // namespace
 
 void launch_tree(dzs_ctx* c) {
-  c->launches += 6;
+  c->launches += 5;
   Buffers& B = c->B;
   // the Morton cell table (also the PM tiles')
   launch_cell_start(c);
@@ -365,8 +370,7 @@ void launch_tree(dzs_ctx* c) {
   int32_t* cfirst = B.cfirst;         // [node_cap]
   k_tree_count<<<(unsigned)ntiles, kTreeTile, 0, c->stream>>>(B.n, B.key, c->P.leaf_bucket, c->P.walk_group, info,
                                                               tcount, ntiles);
-  k_tree_scan<<<kCols, 1024, 0, c->stream>>>(tcount, ntiles, B.lvl_count);
-  k_tree_totals<<<1, 32, 0, c->stream>>>(B.lvl_count, c->node_cap, B.counters, B.err);
+  k_tree_scan<<<kCols, 1024, 0, c->stream>>>(tcount, ntiles, B.lvl_count, c->node_cap, B.counters, B.err);
   k_tree_nodes<<<(unsigned)ntiles, kTreeTile, 0, c->stream>>>(B.n, c->cap, B.key, B.u, info, tcount, ntiles,
                                                               B.lvl_count, B.cell_start, c->cell_depth, c->P.leaf_bucket,
                                                               B.nodes, cfirst, B.parent, B.groups);

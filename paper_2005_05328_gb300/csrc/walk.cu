@@ -482,15 +482,23 @@ __device__ __forceinline__ float radius_of<float>(unsigned long long b) { return
 template <>
 __device__ __forceinline__ double radius_of<double>(unsigned long long b) { return __longlong_as_double((long long)b); }
 
-// per-step walk inputs: packed particle entries (position, G m / s^2) and spline
+// per-step walk inputs: empty frontier tables, packed particle entries (position, G m / s^2) and spline
 // radius, node spline radius
 template <class R>
 __global__ void k_walk_prep(const int32_t* __restrict__ d_n, int64_t cap, const uint32_t* __restrict__ u,
                             const uint32_t* __restrict__ k, const int32_t* __restrict__ lvl,
                             const Node* __restrict__ nodes, Entry<R>* __restrict__ pm,
                             R* __restrict__ ph, R* __restrict__ nh, R gm0, R h0,
-                            unsigned long long* __restrict__ hmax_bits) {
+                            unsigned long long* __restrict__ hmax_bits, int32_t* __restrict__ ftab, int64_t cells,
+                            int32_t* __restrict__ ftabF, uint8_t* __restrict__ fspanF, int64_t cellsF) {
   const int64_t n = *d_n;
+  // the frontier tables start empty
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < cells; q += (int64_t)gridDim.x * blockDim.x)
+    ftab[q] = -1;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < cellsF; q += (int64_t)gridDim.x * blockDim.x) {
+    ftabF[q] = -1;
+    fspanF[q] = 0;
+  }
   int64_t nn = 0;
   for (int j = 0; j <= kMaxLevel; ++j) nn += lvl[j];
   const int64_t m = n > nn ? n : nn;
@@ -1021,20 +1029,20 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
   C.h0 = (R)(2.8 * c->eps0 / s);
   unsigned long long* hmax_slot = (unsigned long long*)(c->B.counters + 24);
   C.hmax = hmax_slot;
-  cudaMemsetAsync(hmax_slot, 0, sizeof(uint64_t), c->stream);
-  k_walk_prep<R><<<grid_for(c->node_cap), kThreads, 0, c->stream>>>(c->B.n, c->cap, c->B.u, c->B.k, c->B.lvl_count,
-                                                                     c->B.nodes, pm, ph, nh, C.gm0, C.h0, hmax_slot);
+  const int64_t cells_f0 = C.front > 0 && tree ? (int64_t)1 << (3 * C.front) : 0;
+  const int64_t cells_F0 = cells_f0 > 0 && C.frontF > 0 ? (int64_t)1 << (3 * C.frontF) : 0;
+  // (the tree build cleared hmax_slot and the work counter)
+  k_walk_prep<R><<<grid_for(c->node_cap), kThreads, 0, c->stream>>>(
+      c->B.n, c->cap, c->B.u, c->B.k, c->B.lvl_count, c->B.nodes, pm, ph, nh, C.gm0, C.h0, hmax_slot, c->B.iscan,
+      cells_f0, (int32_t*)C.ftabF, (uint8_t*)C.fspanF, cells_F0);
   if (C.front > 0 && tree) {
     const int64_t cells = (int64_t)1 << (3 * C.front);
     c->launches += 1;
-    cudaMemsetAsync(c->B.iscan, 0xff, sizeof(int32_t) * cells, c->stream);
     k_front_fill<<<grid_for(cells, kThreads, 4), kThreads, 0, c->stream>>>(c->B.lvl_count, c->B.nodes, C.front,
                                                                                c->B.iscan);
     if (C.frontF > 0) {
       const int64_t cellsF = (int64_t)1 << (3 * C.frontF);
       c->launches += 1;
-      cudaMemsetAsync((void*)C.ftabF, 0xff, sizeof(int32_t) * cellsF, c->stream);
-      cudaMemsetAsync((void*)C.fspanF, 0, (size_t)cellsF, c->stream);
       FarMax fm;
       const double skip_r = std::sqrt((double)C.skip_d2) * (1.0 + 1e-12);
       for (int l = 0; l <= kMaxLevel; ++l) {
@@ -1067,7 +1075,6 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->dev);
   int grid = (per_sm > 0 ? per_sm : 1) * (nsm > 0 ? nsm : 1);
   unsigned int* next = (unsigned int*)(c->B.counters + 6);
-  cudaMemsetAsync(next, 0, sizeof(unsigned int), c->stream);
   kern<<<grid, kWarps * 32, sm, c->stream>>>(c->B.groups, c->B.counters, next, c->B.nodes, nh, c->cap, pm, ph, (R*)c->B.p, (R*)c->B.g, C, c->B.err,
                                                   (unsigned long long*)(c->B.counters + 4), c->B.wlen);
 }
