@@ -34,9 +34,10 @@
 // walk compares integers only (FP32 sums decide unless within 2^-20 of a
 // threshold, where the uint64 sum decides) and builds the same interaction
 // set as the CPU reference, with no FP64 in the traversal.
-// The list lives in shared memory and is evaluated between rounds, when it
-// holds more than 172 entries (a round adds at most 32 monopoles and the
-// leaves that fit; leaves that do not fit wait on the stack).  A group of c
+// Opened leaves queue their particles, and whole batches of 32 are tested and
+// listed.  The list lives in shared memory and is evaluated between rounds and
+// batches, when it holds more than 204 entries (either adds at most 32).  A
+// group of c
 // particles puts every lane to work: lane -> particle m = lane mod c, the
 // S_m lanes of particle m each taking every S_m-th pair of entries; the lanes
 // of a particle are combined by a fixed shuffle tree (the result is
@@ -47,7 +48,12 @@
 // instructions; FP64 reads T(r) / r^3 from a table of polynomials in r^2.
 // Walk of the 128^3 / mesh 256 set, early (30% of listed pairs in range), late,
 // and of 256^3 / mesh 256 (75%): bit-masked or guarded scalar evaluation 2.72,
-// 0.69, 42.1 ms, paired 2.47, 0.60, 34.0 ms.
+// 0.69, 42.1 ms, paired 2.47, 0.60, 34.0 ms.  The walk is bound by issue slots
+// (71% used): of 2.4 ms early, evaluation took 0.63, listing leaf particles 0.55,
+// node rounds 0.87, the rest (start windows, group fetch, closing kick) 0.4.
+// Queued leaf particles and the COM-first node test: 2.41, 0.57, 33.9 -> 2.30,
+// 0.56, 31.2 ms.  Walking two sibling groups together took 2.58 and 39.5 ms (39%
+// fewer rounds, but the shared list has a third more pairs).
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -64,6 +70,10 @@ namespace {
 constexpr int kWarps = 4;
 constexpr int kStack = 512;
 constexpr int kList = 236;
+// particles of opened leaves waiting to be listed: 31 left over from the last
+// batch and 32 leaves of 8 (larger buckets: leaves that do not fit go back on the
+// stack); 7 blocks' shared memory would hold 300
+constexpr int kQueue = 288;
 
 // Q(t) power-series coefficients, t = 2 x / 2.5 - 1; FP32 rel. error 3.32e-07
 // (generated by gen_split_poly.py)
@@ -156,10 +166,12 @@ struct __align__(16) WalkSmem<float> {
   float x[kWarps][kRow], y[kWarps][kRow], z[kWarps][kRow], m[kWarps][kRow];
   float h[kWarps][kRow];  // spline radius 2.8 eps of the entry (lattice units)
   int32_t stack[kWarps][kStack];
+  int32_t queue[kWarps][kQueue];  // particles of opened leaves
 };
 template <>
 struct WalkSmem<double> {
   int32_t stack[kWarps][kStack];
+  int32_t queue[kWarps][kQueue];
   LEntry<double> e[kWarps][kList];
   double h[kWarps][kList];
 };
@@ -207,6 +219,7 @@ struct WalkConst {
   float open_lo[kMaxLevel + 1], open_hi[kMaxLevel + 1];
   int B;
   int close;
+  int wide_open;     // touching implies open at every level
   int tree;
   int front;                  // frontier depth f (0: start at the root)
   const int32_t* ftab;        // [2^f]^3 row-major: node of each depth-f cell, -1 if empty
@@ -646,7 +659,7 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
       const R hi = ph[i];
       R ax = 0, ay = 0, az = 0;
       if (C.tree) {
-        int top = 0, len = 0, glen = 0;
+        int top = 0, len = 0, glen = 0, pend = 0;
         bool started = false;
         if (C.frontF > 0 && glevel >= C.frontF - 1) {
           // the depth-F nodes (or leaves above F) of the cells within r_cut of
@@ -730,10 +743,31 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
     len = 0;                                                                 \
     __syncwarp();                                                            \
   } while (0)
-        while (top > 0) {
-          // the list is evaluated only here, between rounds (a round adds at
-          // most 32 monopoles and the leaves that fit; the others wait)
-          if (len > kList - 64) DZS_WALK_FLUSH();
+        for (;;) {
+          // the list is evaluated only here: a round adds at most 32 monopoles,
+          // a batch at most 32 particles
+          if (len > kList - 32) DZS_WALK_FLUSH();
+          // a full batch of opened leaves' particles, or the last one: a
+          // particle farther than r_cut from the group cube acts on none of the
+          // group's particles and is not listed
+          if (pend >= 32 || (top == 0 && pend > 0)) {
+            const int nb = pend < 32 ? pend : 32;
+            pend -= nb;
+            bool take = false;
+            Entry<R> E;
+            R hj = 0;
+            if (lane < nb) {
+              const int j = sm.queue[w][pend + lane];
+              E = pm[j];
+              hj = ph[j];  // loaded beside the entry, before the distance test
+              take = near_group(E.x, E.y, E.z, cg, hg, C);
+            }
+            const unsigned tm = __ballot_sync(0xffffffffu, take);
+            if (take) put_entry(sm, w, len + __popc(tm & lt), make_entry(E.x, E.y, E.z, E.m, cg), hj);
+            len += __popc(tm);
+            continue;
+          }
+          if (top == 0) break;
           const int npop = top < 32 ? top : 32;
           if (kDiag) {
             ntests += npop;
@@ -749,55 +783,47 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
             nd = nodes[ni];
             nhi = nh[ni];  // the node's softening, loaded beside the node
             const int nlevel = (int)(nd.meta & 0xff);
-            // 32-bit gaps (half extents: group hg <= 2^31, node hn <= 2^30 below
-            // the root, so hg + hn < 2^32); squared sums in FP32 decide unless
-            // they fall within 2^-20 of the exact integer threshold, where the
-            // uint64 sum decides -- the same decision as the integer rule
-            uint32_t gp[3], dmv[3];
-            float d2f = 0.f, c2f = 0.f;
+            // squared distance of the COM to the group cube, 32-bit gaps and an
+            // FP32 sum that decides unless it falls within 2^-20 of the exact
+            // integer threshold, where the uint64 sum decides -- the same
+            // decision as the integer rule
             const uint32_t cm[3] = {nd.comx, nd.comy, nd.comz};
-            // cube centre from the COM (inside the cube) and the level
-            const uint32_t hn = 1u << (31 - nlevel), cmask = ~((hn << 1) - 1u);
-            const uint32_t cn[3] = {(cm[0] & cmask) | hn, (cm[1] & cmask) | hn, (cm[2] & cmask) | hn};
-            // gap = max(|dc|, h) - h; the root touches everything (h = max)
-            const uint32_t h = nlevel == 0 ? 0xffffffffu : hg + (1u << (31 - nlevel));
+            uint32_t dmv[3];
+            float c2f = 0.f;
 #pragma unroll
             for (int a3 = 0; a3 < 3; ++a3) {
-              const uint32_t dc = (uint32_t)abs((int32_t)(cn[a3] - cg[a3]));
-              const uint32_t gap = max(dc, h) - h;
-              gp[a3] = gap;
-              d2f = fmaf((float)gap, (float)gap, d2f);
               const uint32_t mc = (uint32_t)abs((int32_t)(cm[a3] - cg[a3]));
-              const uint32_t dm = max(mc, hg) - hg;
-              dmv[a3] = dm;
-              c2f = fmaf((float)dm, (float)dm, c2f);
+              dmv[a3] = max(mc, hg) - hg;
+              c2f = fmaf((float)dmv[a3], (float)dmv[a3], c2f);
             }
-            const bool touch = (gp[0] | gp[1] | gp[2]) == 0u;
-            bool keep = touch;
-            if (!touch) {
-              if (d2f <= C.skip_lo)
-                keep = true;
-              else if (d2f < C.skip_hi)
-                keep = exact_d2(gp) <= C.skip_d2;
-            }
-            if (keep) {
-              bool open = touch;
-              if (!open) {
-                if (c2f <= C.open_lo[nlevel])
-                  open = true;
-                else if (c2f < C.open_hi[nlevel])
-                  open = exact_d2(dmv) <= C.open_d2[nlevel];
+            // an accepted monopole farther than r_cut from the group cube acts on
+            // none of its particles: not listed
+            const bool near = c2f <= C.skip_lo || (c2f < C.skip_hi && exact_d2(dmv) <= C.skip_d2);
+            bool open = c2f <= C.open_lo[nlevel] || (c2f < C.open_hi[nlevel] && exact_d2(dmv) <= C.open_d2[nlevel]);
+            bool keep = near;
+            // the cube gap decides only where the COM is beyond r_cut and yet close
+            // enough to open (always, when touching may open what the COM does not)
+            if (!C.wide_open || (open && !near)) {
+              // half extents: group hg <= 2^31, node hn <= 2^30 below the root, so
+              // hg + hn < 2^32; cube centre from the COM (inside the cube) and the
+              // level; gap = max(|dc|, h) - h; the root touches everything (h = max)
+              const uint32_t hn = 1u << (31 - nlevel), cmask = ~((hn << 1) - 1u);
+              const uint32_t h = nlevel == 0 ? 0xffffffffu : hg + hn;
+              uint32_t gp[3];
+              float d2f = 0.f;
+#pragma unroll
+              for (int a3 = 0; a3 < 3; ++a3) {
+                const uint32_t dc = (uint32_t)abs((int32_t)(((cm[a3] & cmask) | hn) - cg[a3]));
+                gp[a3] = max(dc, h) - h;
+                d2f = fmaf((float)gp[a3], (float)gp[a3], d2f);
               }
-              if (!open) {
-                // an accepted monopole farther than r_cut from the group cube
-                // acts on none of its particles: not listed
-                acc = c2f <= C.skip_lo || (c2f < C.skip_hi && exact_d2(dmv) <= C.skip_d2);
-              } else if (nd.child < 0) {
-                leaf = true;
-              } else {
-                inner = true;
-              }
+              const bool touch = (gp[0] | gp[1] | gp[2]) == 0u;
+              keep = touch || d2f <= C.skip_lo || (d2f < C.skip_hi && exact_d2(gp) <= C.skip_d2);
+              open = open || touch;
             }
+            acc = near && !open;
+            leaf = keep && open && nd.child < 0;
+            inner = keep && open && nd.child >= 0;
           }
           // accepted monopoles (at most 32 this round)
           unsigned am = __ballot_sync(0xffffffffu, acc);
@@ -806,74 +832,47 @@ __global__ void __launch_bounds__(kWarps * 32, sizeof(R) == 4 ? 7 : 5) k_walk(
             put_entry(sm, w, pos, make_entry(nd.comx, nd.comy, nd.comz, C.gm0 * (R)nd.mass, cg), nhi);
           }
           len += __popc(am);
-          // children of opened inner nodes onto the stack
-          // one scan for both counts: children (<= 8 per lane, total < 2^16) in
-          // the low half, leaf particles (<= B <= 14 per lane) in the high half
+          // one scan for both counts: children of opened inner nodes (<= 8 per
+          // lane, total < 2^16) in the low half, particles of opened small leaves
+          // (<= B <= 14 per lane) in the high half
           int nch = inner ? (int)((nd.meta >> 8) & 0xff) : 0;
           int lc = (leaf && nd.count <= C.B) ? nd.count : 0;
-          const int both = warp_incl_scan(nch | (lc << 16));
-          int ex = (both & 0xffff) - nch;
-          int tot = __shfl_sync(0xffffffffu, both & 0xffff, 31);
-          const int incl = both >> 16;
+          const int incl = warp_incl_scan(nch | (lc << 16));
+          int tot = __shfl_sync(0xffffffffu, incl, 31), items = tot >> 16;
+          tot &= 0xffff;
           if (top + tot > kStack) {
             if (lane == 0) atomicOr(err, kErrStack);
             nch = 0;
             tot = 0;
           }
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (q < nch) sm.stack[w][top + ex + q] = nd.child + q;
+          const int top0 = top;
           top += tot;
-          if (kDiag) maxtop = top > maxtop ? top : maxtop;
-          // particles of opened small leaves, copied cooperatively (item t of
-          // the round belongs to the lane whose inclusive end first exceeds t);
-          // a particle farther than r_cut from the group cube acts on none of
-          // the group's particles and is not listed
-          // leaves whose particles do not fit in the list this round go back
-          // on the stack (the inclusive ends grow with the lane, so the ones
-          // that fit are a prefix); after the next evaluation they fit
-          const int room = kList - len;
-          const bool defer = lc > 0 && incl > room;
-          const unsigned dm = __ballot_sync(0xffffffffu, defer);
-          if (dm) {
+          // leaves whose particles do not fit in the queue go back on the stack
+          // (the inclusive ends grow with the lane: the ones that fit are a prefix)
+          if (pend + items > kQueue) {
+            const bool fits = pend + (incl >> 16) <= kQueue, defer = lc > 0 && !fits;
+            const unsigned dm = __ballot_sync(0xffffffffu, defer);
+            items = (int)__reduce_max_sync(0xffffffffu, fits ? (unsigned)(incl >> 16) : 0u);
             if (top + __popc(dm) > kStack) {
               if (lane == 0) atomicOr(err, kErrStack);
-            } else if (defer) {
-              sm.stack[w][top + __popc(dm & lt)] = ni;
+            } else {
+              if (defer) sm.stack[w][top + __popc(dm & lt)] = ni;
+              top += __popc(dm);
             }
-            top += top + __popc(dm) > kStack ? 0 : __popc(dm);
             if (defer) lc = 0;
           }
-          // items of the leaves that stay: the largest inclusive end within
-          // the room (lanes past a deferred leaf carry its items in incl)
-          const int totl = (int)__reduce_max_sync(0xffffffffu, (unsigned)(incl <= room ? incl : 0));
-          // item t of the owner lane is particle jbase_owner + t
-          const int jbase = leaf ? nd.start - (incl - lc) : 0;
-          for (int b0 = 0; b0 < totl; b0 += 32) {
-            int t = b0 + lane;
-            int src = 0;
+          // an inner node's children onto the stack, a leaf's particles into the queue
+          {
+            const int cn = inner ? nch : lc, v = inner ? nd.child : nd.start;
+            int32_t* const dst =
+                inner ? &sm.stack[w][top0 + (incl & 0xffff) - nch] : &sm.queue[w][pend + (incl >> 16) - lc];
 #pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-              int v = __shfl_sync(0xffffffffu, incl, src + step - 1);
-              if (v <= t) src += step;
-            }
-            const int jb = __shfl_sync(0xffffffffu, jbase, src);
-            bool take = false;
-            Entry<R> E;
-            R hj = 0;
-            if (t < totl) {
-              const int64_t j = (int64_t)jb + t;
-              E = pm[j];
-              hj = ph[j];  // loaded beside the entry, before the distance test
-              take = near_group(E.x, E.y, E.z, cg, hg, C);
-            }
-            const unsigned tm = __ballot_sync(0xffffffffu, take);
-            if (take) {
-              const int pos = len + __popc(tm & lt);
-              put_entry(sm, w, pos, make_entry(E.x, E.y, E.z, E.m, cg), hj);
-            }
-            len += __popc(tm);
+            for (int q = 0; q < 8; ++q)
+              if (q < cn) dst[q] = v + q;
+            for (int q = 8; q < cn; ++q) dst[q] = v + q;
           }
+          pend += items;
+          if (kDiag) maxtop = top > maxtop ? top : maxtop;
           __syncwarp();
           // big leaves (depth 21, more than B particles): stream through
           unsigned bm = __ballot_sync(0xffffffffu, leaf && nd.count > C.B);
@@ -978,6 +977,11 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
     C.open_hi[l] = hi_of(C.open_d2[l]);
   }
   C.B = c->P.leaf_bucket;
+  // a node whose cube touches the group's has its COM within sqrt(3) l of the
+  // group cube: with every threshold at least that, the COM decides alone
+  C.wide_open = 1;
+  for (int l = 0; l <= kMaxLevel; ++l)
+    if (C.open_d2[l] < 3ull << (l ? 64 - 2 * l : 62)) C.wide_open = 0;
   C.close = close_kick ? 1 : 0;
   C.tree = tree ? 1 : 0;
   // frontier depth: every depth above it never accepts (a non-skipped node's
