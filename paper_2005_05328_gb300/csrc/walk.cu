@@ -1096,6 +1096,12 @@ void fill_ztab(double (*tab)[kZDeg + 1]) {
       cheb[j][p] = j == 0 ? (p == 0 ? 1.0L : 0.0L)
                  : j == 1 ? (p == 1 ? 1.0L : 0.0L)
                           : (p > 0 ? 2.0L * cheb[j - 1][p - 1] : 0.0L) - cheb[j - 2][p];
+  ld to_mono[n][n] = {};  // node values -> Chebyshev coefficients -> powers
+  for (int j = 0; j < n; ++j)
+    for (int k = 0; k < n; ++k) {
+      const ld a = cosl(pi * j * (k + 0.5L) / n) * (j == 0 ? 1.0L : 2.0L) / n;
+      for (int p = 0; p <= j; ++p) to_mono[p][k] += cheb[j][p] * a;
+    }
   for (int c = 0; c < kZCells; ++c) {
     const ld width = ldexpl(1.0L / kZSub, kZLo + c / kZSub), half = 0.5L * width;
     const ld mid = ldexpl(1.0L, kZLo + c / kZSub) + width * (c % kZSub) + half;
@@ -1104,12 +1110,8 @@ void fill_ztab(double (*tab)[kZDeg + 1]) {
       const ld z = mid + half * node[k], x = sqrtl(z);
       f[k] = (erfcl(x) + tsp * x * expl(-z)) / (z * x);
     }
-    for (int j = 0; j < n; ++j) {
-      ld a = 0.0L;
-      for (int k = 0; k < n; ++k) a += f[k] * cosl(pi * j * (k + 0.5L) / n);
-      a *= (j == 0 ? 1.0L : 2.0L) / n;
-      for (int p = 0; p <= j; ++p) mono[p] += a * cheb[j][p];
-    }
+    for (int p = 0; p < n; ++p)
+      for (int k = 0; k < n; ++k) mono[p] += to_mono[p][k] * f[k];
     ld scale = 1.0L;
     for (int p = 0; p < n; ++p, scale /= half) tab[c][p] = (double)(mono[p] * scale);
   }
