@@ -3,11 +3,10 @@ the walk group bound G, the leaf size B, theta, the mesh and every other
 parameter that changes a result stay as given).
 
 Knobs:
-  - walk_eval: how the tree walk evaluates its interaction lists (a range-test
-    pass then force arithmetic for the pairs within r_cut, or one guarded
-    pass).  Both evaluate the same pairs in the same order, so results are
-    identical; only the time differs, with the group size against r_cut and
-    with clustering.
+  - walk_eval: how the tree walk evaluates its interaction lists.  The walk has
+    one way of evaluating them (two entries at a time, out-of-range ones
+    dropped by a select), which every value selects: results are identical and
+    the candidates' times differ by noise only.
   - host_threads, steps_per_slice of the serving loop (dzs_serve): how many
     host threads issue the mocks' kernels and how many steps each slice
     enqueues.
