@@ -60,11 +60,11 @@ STAGE_BYTES = {
 # the implementation's own bytes per step (what its kernels read and write,
 # counted from the code), reported beside the algorithmic bytes
 IMPL_BYTES = {
-    "kick_drift": lambda n, m3: 90 * n,
-    "sort": lambda n, m3: 326 * n,
-    "merge": lambda n, m3: 194 * n,
+    "kick_drift": lambda n, m3: 70 * n,
+    "sort": lambda n, m3: 270 * n,
+    "merge": lambda n, m3: 186 * n,
     "tree": lambda n, m3: 95 * n,
-    "pm": lambda n, m3: 16.0 * m3 + 40 * n,
+    "pm": lambda n, m3: 16.8 * m3 + 67 * n,
     "fft": lambda n, m3: 40.3 * m3,
 }
 
