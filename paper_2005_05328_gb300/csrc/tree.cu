@@ -218,9 +218,10 @@ __global__ void __launch_bounds__(kTreeTile) k_tree_nodes(
       if (lane >= o) inc += up;
     }
     // nodes of the shallower depths; groups have a numbering of their own; -1:
-    // no tree (over capacity)
-    if (lane < kCols) base[lane] = t + (lane <= kMaxLevel ? inc - v : 0);
-    if (lane == 31 && inc == 0) base[0] = -1;
+    // no tree (over capacity).  One lane writes each slot: the guard below keeps
+    // every block off the node array and must not hang on the order of two stores
+    const bool none = __shfl_sync(kFull, inc, 31) == 0;
+    if (lane < kCols) base[lane] = none ? -1 : t + (lane <= kMaxLevel ? inc - v : 0);
   }
   for (int q = threadIdx.x; q < kTreeTile + kHalo; q += kTreeTile) ks[q] = t0 + q < n ? key[t0 + q] : ~0ull;
   for (int q = threadIdx.x; q < (kTreeTile / 32) * kCols; q += kTreeTile) (&wcnt[0][0])[q] = 0;
