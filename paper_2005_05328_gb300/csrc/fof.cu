@@ -255,7 +255,7 @@ __global__ void k_fof_labels(const int32_t* __restrict__ d_n, const int32_t* __r
 // (halo records, nmin >= 2 keeps them within 32 bytes per particle), the PM
 // cell table (cells of depth `depth`).  Leaves the halo count in n[2].
 void launch_fof(dzs_ctx* c, int depth, uint64_t T, int nmin, int64_t* d_label, dzs_halo** d_halos) {
-  c->launches += 8;
+  c->launches += d_label ? 7 : 6;  // (the cell table and the scan count their own)
   Buffers& B = c->B;
   const int64_t cap = c->cap;
   char* pre = (char*)B.prefix;

@@ -113,6 +113,7 @@ __global__ void k_ics_finish(int64_t n, int64_t cap, const uint32_t* __restrict_
 }  // namespace
 
 void launch_ics(dzs_ctx* c) {
+  c->launches += 1 + 3 + 1 + 3 * 5 + 1;  // noise, FFT, delta, per axis psi, inverse FFT and placement, finish
   const int n1 = c->n1;
   const int64_t n = c->N0, hn = n1 / 2 + 1;
   const int64_t nspec = (int64_t)n1 * n1 * hn;

@@ -560,6 +560,9 @@ void pm_deposit(dzs_ctx* c) {
       B.cell_start, B.n, (const R*)B.cicw, M, (R*)B.rho, inv_nbar);
 }
 
+// kernels of pm_deposit itself (launch_sort_keys counts the cell sort's)
+int deposit_kernels(const dzs_ctx* c) { return !c->mesh_pow2 ? 4 : tile_mesh(c) ? 1 : 2; }
+
 template <class R>
 void pm_fft(dzs_ctx* c) {
   Buffers& B = c->B;
@@ -776,7 +779,9 @@ void pk_impl(dzs_ctx* c, int nbins, double* d_part, double* d_out, double shot) 
 // [nbins][3]; d_part is scratch of M * nbins * 3 doubles.  The state must be
 // Morton-sorted with valid keys.
 void launch_pk(dzs_ctx* c, int nbins, double* d_part, double* d_out, double shot) {
-  c->launches += c->mesh_pow2 ? 8 : 16;
+  // deposit, FFT (3), shells, planes, final; the cell table and the mesh's cell
+  // sort count their own
+  c->launches += deposit_kernels(c) + 6;
   if (c->fp64)
     pk_impl<double>(c, nbins, d_part, d_out, shot);
   else
@@ -804,7 +809,7 @@ void launch_cells(dzs_ctx* c, int depth) {
 void launch_cell_start(dzs_ctx* c) { launch_cells(c, c->cell_depth); }
 
 void launch_pm_deposit(dzs_ctx* c) {
-  c->launches += !c->mesh_pow2 ? 9 : tile_mesh(c) ? 1 : 2;
+  c->launches += deposit_kernels(c);
   if (c->fp64)
     pm_deposit<double>(c);
   else

@@ -101,6 +101,7 @@ __global__ void k_chunk_scan(const int32_t* __restrict__ in, const int32_t* d_n,
 }  // namespace
 
 void exclusive_scan_i32(dzs_ctx* c, const int32_t* in, int32_t* out, const int32_t* d_n, int64_t cap) {
+  c->launches += 3;
   int nchunks = (int)((cap + kChunk) / kChunk);  // covers index cap itself
   k_chunk_totals<<<nchunks, 256, 0, c->stream>>>(in, d_n, c->B.blocksum);
   k_scan_totals<<<1, 1024, 0, c->stream>>>(c->B.blocksum, nchunks);

@@ -314,6 +314,7 @@ void launch_diagnostics(dzs_ctx* c) {
 }
 
 void launch_to_double(dzs_ctx* c, const void* src, int64_t count, double* dst) {
+  c->launches += c->fp64 ? 0 : 1;
   if (c->fp64)
     cudaMemcpyAsync(dst, src, count * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
   else
@@ -321,6 +322,7 @@ void launch_to_double(dzs_ctx* c, const void* src, int64_t count, double* dst) {
 }
 
 void launch_from_double(dzs_ctx* c, const double* src, int64_t count, void* dst) {
+  c->launches += c->fp64 ? 0 : 1;
   if (c->fp64)
     cudaMemcpyAsync(dst, src, count * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
   else
