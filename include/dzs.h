@@ -550,6 +550,11 @@ DZS_API dzs_status dzs_twin_displacement(dzs_ctx* a, dzs_ctx* b, const double* e
  * call returns DZS_ENOMEM and frees what it had allocated. */
 DZS_API void dzs_debug_fail_alloc(int32_t k);
 
+/* Test hook: polls a waiting block of the radix sort makes of an earlier
+ * block's published counts before it counts those keys itself (a negative
+ * value restores the default, about a second).  Results do not depend on it. */
+DZS_API void dzs_debug_sort_look(int32_t polls);
+
 /* Message of the last failure on this context (valid until the next call).
  * c may be NULL (then: the last dzs_create failure of this thread). */
 DZS_API const char* dzs_last_error(const dzs_ctx* c);

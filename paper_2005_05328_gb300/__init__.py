@@ -35,7 +35,7 @@ EXPORTED = ["dzs_params_default", "dzs_footprint_bytes", "dzs_create", "dzs_ics"
             "dzs_run_stages", "dzs_lightcone_drain", "dzs_pipeline", "dzs_step_result", "dzs_lightcone_drain_step",
             "dzs_destroy", "dzs_get_count", "dzs_get_state",
             "dzs_set_state", "dzs_accel", "dzs_merge_only", "dzs_diagnostics", "dzs_get_tables",
-            "dzs_get_mesh", "dzs_get_counters", "dzs_get_walk_counters", "dzs_walk_lists", "dzs_measure_fp32_peaks", "dzs_debug_fail_alloc", "dzs_twin_displacement", "dzs_batch_create", "dzs_batch_step",
+            "dzs_get_mesh", "dzs_get_counters", "dzs_get_walk_counters", "dzs_walk_lists", "dzs_measure_fp32_peaks", "dzs_debug_fail_alloc", "dzs_debug_sort_look", "dzs_twin_displacement", "dzs_batch_create", "dzs_batch_step",
             "dzs_batch_synchronize", "dzs_batch_destroy", "dzs_set_profiling", "dzs_get_profile",
             "dzs_morton_sort_noalloc", "dzs_checkpoint_bytes", "dzs_checkpoint", "dzs_restore",
             "dzs_step_until", "dzs_observe_enable", "dzs_observe_add_records", "dzs_skymap_get",
@@ -128,6 +128,7 @@ def load(path: str = LIB_PATH):
         "dzs_walk_lists": [vp, vp, vp, vp, sz, C.POINTER(sz)],
         "dzs_measure_fp32_peaks": [i32, i32, C.POINTER(C.c_double), C.POINTER(C.c_double)],
         "dzs_debug_fail_alloc": [i32],
+        "dzs_debug_sort_look": [i32],
         "dzs_batch_create": [vp, i32, i32, C.POINTER(vp)], "dzs_batch_step": [vp, i32, i32, vp],
         "dzs_batch_synchronize": [vp], "dzs_batch_destroy": [vp],
         "dzs_twin_displacement": [vp, vp, vp, i32, vp, vp, C.POINTER(C.c_double)], "dzs_set_profiling": [vp, i32], "dzs_get_profile": [vp, vp, vp],
@@ -147,6 +148,7 @@ def load(path: str = LIB_PATH):
     L.dzs_morton_sort_noalloc.argtypes = [vp, sz, vp, vp, vp]
     L.dzs_morton_sort_noalloc.restype = C.c_int
     L.dzs_debug_fail_alloc.restype = None
+    L.dzs_debug_sort_look.restype = None
     L.dzs_last_error.argtypes = [vp]
     L.dzs_last_error.restype = C.c_char_p
     _lib = L
@@ -374,6 +376,11 @@ class Batch:
 def dzs_debug_fail_alloc(k):
     """test hook: the k-th device allocation from now on fails (0: off)"""
     load().dzs_debug_fail_alloc(int(k))
+
+
+def dzs_debug_sort_look(polls):
+    """test hook: polls of the sort's look-back before it counts for itself (< 0: default)"""
+    load().dzs_debug_sort_look(int(polls))
 
 
 def dzs_twin_displacement(ha, hb, edges):

@@ -194,12 +194,8 @@ dzs_status fail(dzs_ctx* c, dzs_status s, const char* what, const char* detail =
 }
 
 dzs_status device_error_status(dzs_ctx* c, uint32_t err) {
-  char buf[160];
-  if (err & kErrSort) {
-    snprintf(buf, sizeof buf, "a bounded device wait of the sort gave up (error word 0x%x)", err);
-    return fail(c, DZS_ETIMEOUT, buf);
-  }
   if (err & (kErrNodes | kErrStack | kErrGroups)) {
+    char buf[160];
     snprintf(buf, sizeof buf, "device buffer overflow (error word 0x%x)", err);
     return fail(c, DZS_EOVERFLOW, buf);
   }

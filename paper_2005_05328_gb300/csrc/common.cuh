@@ -21,8 +21,6 @@ enum : uint32_t {
   kErrStack = 2u,    // walk stack overflow
   kErrRing = 4u,     // lightcone ring full (records dropped)
   kErrGroups = 8u,   // group capacity exceeded
-  kErrSort = 16u,    // a sort look-back gave up (bounded wait)
-  kErrCell = 32u,    // CIC cell start table inconsistent
 };
 
 // flag bits: bit 0 crossed (public), bit 1 merged (public), bit 2 crossed in

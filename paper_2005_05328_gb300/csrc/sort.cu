@@ -8,6 +8,8 @@
 // block ranks a tile of keys, learns how many keys of each digit the tiles
 // before it hold by looking back over their published counts, and writes the
 // tile.  Ties keep the previous order, so the result is deterministic.
+#include <atomic>
+
 #include "common.cuh"
 
 namespace dzs {
@@ -25,7 +27,9 @@ constexpr int64_t kLargeFrom = 1 << 19;
 // the tile's own count or already the sum over all tiles up to it
 constexpr uint32_t kOwn = 1u << 30, kSum = 2u << 30, kCount = kOwn - 1u;
 constexpr int kLook = 8;
-constexpr int kLookLimit = 1 << 21;  // polls (about a second) before a look-back gives up (error bit)
+// polls (about a second) before a look-back counts the earlier tiles' keys itself
+constexpr int kLookLimit = 1 << 21;
+std::atomic<int> g_look_limit{kLookLimit};
 
 // scratch of a sort (words): digit counts of every pass, a ticket per pass, two
 // tables of status words (a pass fills one and clears the other for the next)
@@ -106,7 +110,10 @@ __device__ __forceinline__ unsigned same_digit(unsigned d, bool valid) {
 }
 
 // One pass.  Tiles are taken by ticket, so every tile before a block's is
-// already held by a running block and the look-back ends.  A warp ranks its
+// already held by a running block and the look-back ends; should a tile not
+// publish within kLookLimit polls, the waiting block counts the digits of the
+// keys before it from the pass's input, which nobody writes: no wait is without
+// an end and no result depends on one.  A warp ranks its
 // own consecutive keys 32 at a time against counters of its own: no block
 // barrier inside the ranking (the tile used to pass four per 256 keys).
 // The tile is placed in shared memory before the look-back, which gives the
@@ -121,7 +128,7 @@ template <int kThr, int kItems>
 __global__ void __launch_bounds__(kThr, 1024 / kThr)
     k_sort_pass(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint64_t* __restrict__ kout,
                 uint32_t* __restrict__ vout, const int32_t* __restrict__ d_n, int pass, uint32_t* __restrict__ scratch,
-                int64_t tiles, uint32_t* __restrict__ err) {
+                int64_t tiles, int look_limit) {
   constexpr int kTile = kThr * kItems, kW = kThr / 32;
   extern __shared__ uint64_t sort_sm[];
   uint64_t* sk = sort_sm;                                           // [kTile] the tile, stably sorted by digit
@@ -137,6 +144,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
   for (int q = t; q < kW * kDigits / 2; q += kThr) reinterpret_cast<uint32_t*>(&wcnt[0][0])[q] = 0;
   __syncthreads();
   const int64_t tile = s_tile, base = tile * kTile;
+  if (tile >= tiles) return;  // never, unless such calls took tickets here
   uint32_t* status = scratch + kOffStatus + (pass & 1 ? tiles * kDigits : 0);
   uint32_t* other = scratch + kOffStatus + (pass & 1 ? 0 : tiles * kDigits);
   if (t < kDigits) other[tile * kDigits + t] = 0;  // the next pass's table
@@ -213,8 +221,8 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
         }
       }
       if (next == back) {
-        if (++polls > kLookLimit) {
-          if (err) atomicOr(err, kErrSort);
+        if (++polls > look_limit) {
+          for (int64_t j = 0; j < (back + 1) * kTile; ++j) prev += ((uint32_t)(kin[j] >> shift) & 0xffu) == (uint32_t)t;
           break;
         }
         __nanosleep(64);
@@ -230,7 +238,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
     const uint64_t kv = sk[q];
     const int d = (int)((kv >> shift) & 0xff);
     const uint32_t pos = gbase[d] + (uint32_t)q - lbase[d];
-    if ((int64_t)pos < n) {  // always, unless the look-back gave up
+    if ((int64_t)pos < n) {  // always, unless calls that share the static scratch overlap
       kout[pos] = kv;
       vout[pos] = sv[q];
     }
@@ -239,7 +247,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
 
 // an even number of passes from bit 0; the result is in ka / va again
 void sort_passes(uint64_t* ka, uint64_t* kb, uint32_t* va, uint32_t* vb, const int32_t* d_n, int64_t cap, int passes,
-                 uint32_t* scratch, uint32_t* err, cudaStream_t st) {
+                 uint32_t* scratch, cudaStream_t st) {
   const int64_t tiles = sort_tiles(cap);
   const bool large = cap >= kLargeFrom;
   auto kern = large ? k_sort_pass<kLargeThreads, kLargeItems> : k_sort_pass<kSmallThreads, kSmallItems>;
@@ -250,8 +258,9 @@ void sort_passes(uint64_t* ka, uint64_t* kb, uint32_t* va, uint32_t* vb, const i
   k_digit_counts<<<grid_for(cap, 2 * kSortThreads, 4), kSortThreads, 0, st>>>(ka, d_n, passes, scratch, tiles);
   uint64_t *kin = ka, *kout = kb;
   uint32_t *vin = va, *vout = vb;
+  const int look = g_look_limit.load(std::memory_order_relaxed);
   for (int pass = 0; pass < passes; ++pass) {
-    kern<<<(unsigned)tiles, threads, sm, st>>>(kin, vin, kout, vout, d_n, pass, scratch, tiles, err);
+    kern<<<(unsigned)tiles, threads, sm, st>>>(kin, vin, kout, vout, d_n, pass, scratch, tiles, look);
     std::swap(kin, kout);
     std::swap(vin, vout);
   }
@@ -288,7 +297,7 @@ size_t sort_scratch_words(int64_t n) {
 // with their indices (identity on input); the result is in ka / va again
 void launch_sort_keys(dzs_ctx* c, uint64_t* ka, uint64_t* kb, uint32_t* va, uint32_t* vb, int passes) {
   c->launches += passes + 1;
-  sort_passes(ka, kb, va, vb, c->B.n, c->cap, passes, c->B.hist, c->B.err, c->stream);
+  sort_passes(ka, kb, va, vb, c->B.n, c->cap, passes, c->B.hist, c->stream);
 }
 
 void launch_sort(dzs_ctx* c) {
@@ -472,9 +481,13 @@ extern "C" dzs_status dzs_morton_sort_noalloc(const uint32_t* d_u, size_t n, uin
   if (cudaPeekAtLastError() != cudaSuccess) return DZS_ECUDA;
   k_keys<<<grid_for((int64_t)n), kThreads, 0, st>>>(count, (int64_t)n, d_u, keyA);
   if (cudaPeekAtLastError() != cudaSuccess) return DZS_ECUDA;
-  sort_passes(keyA, keyB, valA, valB, count, (int64_t)n, kPasses, hist, nullptr, st);
+  sort_passes(keyA, keyB, valA, valB, count, (int64_t)n, kPasses, hist, st);
   if (cudaPeekAtLastError() != cudaSuccess) return DZS_ECUDA;
   if (cudaMemcpyAsync(d_perm, valA, 4 * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return DZS_ECUDA;
   if (d_keys && cudaMemcpyAsync(d_keys, keyA, 8 * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return DZS_ECUDA;
   return DZS_OK;
+}
+
+extern "C" void dzs_debug_sort_look(int32_t polls) {
+  dzs::g_look_limit.store(polls < 0 ? dzs::kLookLimit : polls, std::memory_order_relaxed);
 }
