@@ -18,10 +18,19 @@ namespace {
 constexpr int kSortThreads = 256;
 constexpr int kDigits = 256;
 constexpr int kPasses = 8;
-// tiles: 512 threads x 14 keys (two blocks per SM hold 2.2M keys at once), for
-// fewer keys 256 x 4, spread over more SMs
+// Tiles.  Capacity from 2^19 on: 512 threads with 2, 6 or 14 keys each, the
+// smallest of which one wave holds all keys (two blocks per SM of 152; 14 is what
+// the shared memory of two blocks takes).  The count decides, on the device: DZS
+// shrinks the set under a fixed capacity, and tiles of 14 for every count left
+// most SMs without one (sort stage of 66k / 140k / 300k / 541k / 885k keys in a
+// 128^3 context: 171, 191, 204, 210, 215 us; now 91, 104, 124, 143, 156; 2.1M 247,
+// 250, 16.8M 1510, 1490).  Below 2^19: 256 x 4.
 constexpr int kLargeThreads = 512, kLargeItems = 14, kSmallThreads = 256, kSmallItems = 4;
-constexpr int64_t kLargeFrom = 1 << 19;
+constexpr int kStep1 = 2, kStep2 = 6;
+constexpr int64_t kLargeFrom = 1 << 19, kWave = 2 * 152;
+__host__ __device__ constexpr int tile_items(int64_t n) {
+  return n <= kWave * kLargeThreads * kStep1 ? kStep1 : n <= kWave * kLargeThreads * kStep2 ? kStep2 : kLargeItems;
+}
 
 // status word of a (tile, digit): count in the low 30 bits, and whether it is
 // the tile's own count or already the sum over all tiles up to it
@@ -35,9 +44,12 @@ std::atomic<int> g_look_limit{kLookLimit};
 // tables of status words (a pass fills one and clears the other for the next)
 constexpr int kOffTicket = kPasses * kDigits, kOffStatus = kOffTicket + 32;
 
-inline int64_t sort_tiles(int64_t n) {
-  const int64_t tile = n >= kLargeFrom ? kLargeThreads * kLargeItems : kSmallThreads * kSmallItems;
-  return (n + tile - 1) / tile;
+// most tiles of any count up to cap: a wave of the smaller tiles, the largest
+// tiles beyond
+inline int64_t sort_tiles(int64_t cap) {
+  const int64_t tile = cap >= kLargeFrom ? kLargeThreads * kLargeItems : kSmallThreads * kSmallItems;
+  const int64_t full = (cap + tile - 1) / tile;
+  return cap >= kLargeFrom && full < kWave ? kWave : full;
 }
 // shared memory of a pass: the tile's keys and values, the warps' counters
 constexpr size_t pass_smem(int threads, int items) {
@@ -123,13 +135,16 @@ __device__ __forceinline__ unsigned same_digit(unsigned d, bool valid) {
 // by the look-back and the ranking's instructions (~170 per 32 keys).  Sort
 // stage of 33k / 262k / 2.1M / 16.8M particles with three kernels a pass (digit
 // counts per tile, row scans, scatter): 137, 154, 317, 1850 us; now 63, 103,
-// 230, 1440.
+// 230, 1440.  The keys of a thread are passed over in the three groups of its
+// possible counts, one uniform branch before each; a body per count spilled (16.8M
+// keys 22% slower), a branch per key cost the overlap between keys (2.1M 3%).
 template <int kThr, int kItems>
 __global__ void __launch_bounds__(kThr, 1024 / kThr)
     k_sort_pass(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint64_t* __restrict__ kout,
                 uint32_t* __restrict__ vout, const int32_t* __restrict__ d_n, int pass, uint32_t* __restrict__ scratch,
-                int64_t tiles, int look_limit) {
-  constexpr int kTile = kThr * kItems, kW = kThr / 32;
+                int tiles, int look_limit) {
+  constexpr int kTile = kThr * kItems, kW = kThr / 32;  // the largest tile
+  constexpr bool kVar = kItems == kLargeItems;  // keys per thread by the count
   extern __shared__ uint64_t sort_sm[];
   uint64_t* sk = sort_sm;                                           // [kTile] the tile, stably sorted by digit
   uint32_t* sv = reinterpret_cast<uint32_t*>(sk + kTile);           // [kTile]
@@ -138,25 +153,27 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
   __shared__ uint32_t lbase[kDigits];  // the same within the tile
   __shared__ uint32_t wtot[2][kW];
   __shared__ int s_tile;
-  const int64_t n = *d_n;
+  const int n = *d_n;  // <= 2^27, as every index here
   const int t = threadIdx.x, lane = t & 31, w = t >> 5, shift = 8 * pass;
   if (t == 0) s_tile = (int)atomicAdd(&scratch[kOffTicket + pass], 1u);
   for (int q = t; q < kW * kDigits / 2; q += kThr) reinterpret_cast<uint32_t*>(&wcnt[0][0])[q] = 0;
   __syncthreads();
-  const int64_t tile = s_tile, base = tile * kTile;
-  if (tile >= tiles) return;  // never, unless such calls took tickets here
+  const int items = kVar ? tile_items(n) : kItems, tkeys = kThr * items;
+  const int tile = s_tile, base = tile * tkeys;
+  if (tile >= tiles) return;  // never, unless calls that share the static scratch overlap
   uint32_t* status = scratch + kOffStatus + (pass & 1 ? tiles * kDigits : 0);
   uint32_t* other = scratch + kOffStatus + (pass & 1 ? 0 : tiles * kDigits);
   if (t < kDigits) other[tile * kDigits + t] = 0;  // the next pass's table
   if (base >= n) return;
-  const int tile_n = (int)(n - base < kTile ? n - base : kTile);
+  const int tile_n = min(n - base, tkeys);
   uint64_t kreg[kItems];
   uint32_t vreg[kItems];
   uint16_t rank[kItems];
-  const int64_t i0 = base + w * 32 * kItems + lane;  // the warp's keys are consecutive
+  const int i0 = base + w * 32 * items + lane;  // the warp's keys are consecutive
 #pragma unroll
   for (int s = 0; s < kItems; ++s) {
-    const int64_t i = i0 + s * 32;
+    if (kVar && (s == kStep1 || s == kStep2) && s >= items) break;
+    const int i = i0 + s * 32;
     kreg[s] = i < n ? kin[i] : 0ull;
     vreg[s] = i < n ? (pass == 0 ? (uint32_t)i : vin[i]) : 0u;  // indices start as the identity
   }
@@ -164,6 +181,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int s = 0; s < kItems; ++s) {
+    if (kVar && (s == kStep1 || s == kStep2) && s >= items) break;
     const bool valid = i0 + s * 32 < n;
     const unsigned d = (unsigned)(kreg[s] >> shift) & 0xffu;
     const unsigned peers = same_digit(d, valid);
@@ -193,6 +211,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
   // place the tile while the tiles before it publish their counts
 #pragma unroll
   for (int s = 0; s < kItems; ++s) {
+    if (kVar && (s == kStep1 || s == kStep2) && s >= items) break;
     if (i0 + s * 32 < n) {
       const int d = (int)((kreg[s] >> shift) & 0xff);
       const uint32_t lp = lbase[d] + wcnt[w][d] + rank[s];
@@ -204,12 +223,12 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
   // at a time (one by one, the ~700 tiles of a wave cost as many L2 latencies)
   if (t < kDigits) {
     uint32_t prev = 0;
-    int64_t back = tile - 1;
+    int back = tile - 1;
     for (int polls = 0; back >= 0;) {
       uint32_t v[kLook];
 #pragma unroll
       for (int q = 0; q < kLook; ++q) v[q] = back - q >= 0 ? st[(back - q) * kDigits] : 0u;
-      int64_t next = back;
+      int next = back;
       bool open = true;
 #pragma unroll
       for (int q = 0; q < kLook; ++q) {
@@ -222,7 +241,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
       }
       if (next == back) {
         if (++polls > look_limit) {
-          for (int64_t j = 0; j < (back + 1) * kTile; ++j) prev += ((uint32_t)(kin[j] >> shift) & 0xffu) == (uint32_t)t;
+          for (int j = 0; j < (back + 1) * tkeys; ++j) prev += ((uint32_t)(kin[j] >> shift) & 0xffu) == (uint32_t)t;
           break;
         }
         __nanosleep(64);
@@ -238,7 +257,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
     const uint64_t kv = sk[q];
     const int d = (int)((kv >> shift) & 0xff);
     const uint32_t pos = gbase[d] + (uint32_t)q - lbase[d];
-    if ((int64_t)pos < n) {  // always, unless calls that share the static scratch overlap
+    if (pos < (uint32_t)n) {  // always, unless calls that share the static scratch overlap
       kout[pos] = kv;
       vout[pos] = sv[q];
     }
@@ -260,7 +279,7 @@ void sort_passes(uint64_t* ka, uint64_t* kb, uint32_t* va, uint32_t* vb, const i
   uint32_t *vin = va, *vout = vb;
   const int look = g_look_limit.load(std::memory_order_relaxed);
   for (int pass = 0; pass < passes; ++pass) {
-    kern<<<(unsigned)tiles, threads, sm, st>>>(kin, vin, kout, vout, d_n, pass, scratch, tiles, look);
+    kern<<<(unsigned)tiles, threads, sm, st>>>(kin, vin, kout, vout, d_n, pass, scratch, (int)tiles, look);
     std::swap(kin, kout);
     std::swap(vin, vout);
   }
