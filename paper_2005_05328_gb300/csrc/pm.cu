@@ -623,15 +623,42 @@ __device__ __forceinline__ int mode_bin(int n2) {
   return b;
 }
 
-// |d|^2 added to the pair (hi, lo): FP32 products and sums with their exact
-// remainders (lo collects them), 48 bits altogether; FP64 needs no lo
-__device__ __forceinline__ void add_square(float v, float& hi, float& lo) {
-  const float p = __fmul_rn(v, v), e = __fmaf_rn(v, v, -p);
-  const float s = __fadd_rn(hi, p), t = __fsub_rn(s, hi);
-  lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(p, t)), e));
-  hi = s;
+// |d0|^2 + .. + |d3|^2 in FP64 (the square of an FP32 value is exact there)
+template <class R>
+__device__ __forceinline__ double squares_fp64(const cplx<R> (&d)[4]) {
+  double s = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) s = fma((double)d[q].y, (double)d[q].y, fma((double)d[q].x, (double)d[q].x, s));
+  return s;
 }
-__device__ __forceinline__ void add_square(double v, double& hi, double&) { hi = fma(v, v, hi); }
+
+// a + b = s + (returned remainder), exactly
+__device__ __forceinline__ float two_sum(float a, float b, float& s) {
+  s = __fadd_rn(a, b);
+  const float t = __fsub_rn(s, a);
+  return __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// the same on the FP32 units: products with their exact remainders, summed in three
+// words (hi and lo by exact additions; rest collects what those leave, 2^-48 of hi,
+// rounded to 2^-24 of that).  Largest error over random sums 1.6 units of 2^-53, of
+// the FP64 chain 5.2.  That chain, two conversions and two multiply-adds a clock and
+// SM, took 0.22 ms more at mesh 512 (P(k) 4.54 -> 4.76 ms; three words 4.54, two,
+// which keep 48 bits only, 4.53).  Where a remainder may leave the FP32 range the
+// FP64 sum decides.
+__device__ __forceinline__ double squares(const cplx<float> (&d)[4]) {
+  float hi = 0.f, lo = 0.f, rest = 0.f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float v = q & 1 ? d[q >> 1].y : d[q >> 1].x;
+    const float p = __fmul_rn(v, v), e = __fmaf_rn(v, v, -p);
+    const float t = two_sum(hi, p, hi), r0 = two_sum(lo, t, lo), r1 = two_sum(lo, e, lo);
+    rest = __fadd_rn(rest, __fadd_rn(r0, r1));
+  }
+  if (!(hi >= 0x1p-90f && hi <= 0x1p120f)) return squares_fp64(d);
+  return ((double)hi + (double)lo) + (double)rest;
+}
+__device__ __forceinline__ double squares(const cplx<double> (&d)[4]) { return squares_fp64(d); }
 
 // pairs[s] = number of (ky, kz), signs included, with ky^2 + kz^2 = s
 __global__ void k_pk_shells(int M, int smax, unsigned* __restrict__ pairs) {
@@ -673,19 +700,10 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_plane(const cplx<R>* __restri
       b = mode_bin(n2);
       const bool twoy = ky != 0 && 2 * ky != M;
       const cplx<R> zero = {0, 0};
-      const cplx<R> d0 = spec[(px + ky) * HP + kz], d1 = twox ? spec[(qx + ky) * HP + kz] : zero,
-                    d2 = twoy ? spec[(px + M - ky) * HP + kz] : zero,
-                    d3 = twox && twoy ? spec[(qx + M - ky) * HP + kz] : zero;
-      R hi = 0, lo = 0;
-      add_square(d0.x, hi, lo);
-      add_square(d0.y, hi, lo);
-      add_square(d1.x, hi, lo);
-      add_square(d1.y, hi, lo);
-      add_square(d2.x, hi, lo);
-      add_square(d2.y, hi, lo);
-      add_square(d3.x, hi, lo);
-      add_square(d3.y, hi, lo);
-      v = ((double)hi + (double)lo) * (iw[kx] * iw[ky]) * (kz == 0 || 2 * kz == M ? iw[kz] : 2.0 * iw[kz]);
+      const cplx<R> d[4] = {spec[(px + ky) * HP + kz], twox ? spec[(qx + ky) * HP + kz] : zero,
+                            twoy ? spec[(px + M - ky) * HP + kz] : zero,
+                            twox && twoy ? spec[(qx + M - ky) * HP + kz] : zero};
+      v = squares(d) * (iw[kx] * iw[ky]) * (kz == 0 || 2 * kz == M ? iw[kz] : 2.0 * iw[kz]);
     }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
