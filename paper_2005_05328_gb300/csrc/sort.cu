@@ -9,6 +9,7 @@
 // before it hold by looking back over their published counts, and writes the
 // tile.  Ties keep the previous order, so the result is deterministic.
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -145,6 +146,8 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
                 int tiles, int look_limit) {
   constexpr int kTile = kThr * kItems, kW = kThr / 32;  // the largest tile
   constexpr bool kVar = kItems == kLargeItems;  // keys per thread by the count
+  // at most 2^27 keys; 64 bits where registers allow (20011 keys 3% slower with 32)
+  using I = std::conditional_t<kVar, int, int64_t>;
   extern __shared__ uint64_t sort_sm[];
   uint64_t* sk = sort_sm;                                           // [kTile] the tile, stably sorted by digit
   uint32_t* sv = reinterpret_cast<uint32_t*>(sk + kTile);           // [kTile]
@@ -153,27 +156,28 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
   __shared__ uint32_t lbase[kDigits];  // the same within the tile
   __shared__ uint32_t wtot[2][kW];
   __shared__ int s_tile;
-  const int n = *d_n;  // <= 2^27, as every index here
+  const I n = *d_n;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5, shift = 8 * pass;
   if (t == 0) s_tile = (int)atomicAdd(&scratch[kOffTicket + pass], 1u);
   for (int q = t; q < kW * kDigits / 2; q += kThr) reinterpret_cast<uint32_t*>(&wcnt[0][0])[q] = 0;
   __syncthreads();
-  const int items = kVar ? tile_items(n) : kItems, tkeys = kThr * items;
-  const int tile = s_tile, base = tile * tkeys;
+  const int items = kVar ? tile_items(n) : kItems;
+  const I tkeys = kThr * items;
+  const I tile = s_tile, base = tile * tkeys;
   if (tile >= tiles) return;  // never, unless calls that share the static scratch overlap
   uint32_t* status = scratch + kOffStatus + (pass & 1 ? tiles * kDigits : 0);
   uint32_t* other = scratch + kOffStatus + (pass & 1 ? 0 : tiles * kDigits);
   if (t < kDigits) other[tile * kDigits + t] = 0;  // the next pass's table
   if (base >= n) return;
-  const int tile_n = min(n - base, tkeys);
+  const int tile_n = (int)min(n - base, tkeys);
   uint64_t kreg[kItems];
   uint32_t vreg[kItems];
   uint16_t rank[kItems];
-  const int i0 = base + w * 32 * items + lane;  // the warp's keys are consecutive
+  const I i0 = base + w * 32 * items + lane;  // the warp's keys are consecutive
 #pragma unroll
   for (int s = 0; s < kItems; ++s) {
     if (kVar && (s == kStep1 || s == kStep2) && s >= items) break;
-    const int i = i0 + s * 32;
+    const I i = i0 + s * 32;
     kreg[s] = i < n ? kin[i] : 0ull;
     vreg[s] = i < n ? (pass == 0 ? (uint32_t)i : vin[i]) : 0u;  // indices start as the identity
   }
@@ -223,12 +227,12 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
   // at a time (one by one, the ~700 tiles of a wave cost as many L2 latencies)
   if (t < kDigits) {
     uint32_t prev = 0;
-    int back = tile - 1;
+    I back = tile - 1;
     for (int polls = 0; back >= 0;) {
       uint32_t v[kLook];
 #pragma unroll
       for (int q = 0; q < kLook; ++q) v[q] = back - q >= 0 ? st[(back - q) * kDigits] : 0u;
-      int next = back;
+      I next = back;
       bool open = true;
 #pragma unroll
       for (int q = 0; q < kLook; ++q) {
@@ -241,7 +245,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
       }
       if (next == back) {
         if (++polls > look_limit) {
-          for (int j = 0; j < (back + 1) * tkeys; ++j) prev += ((uint32_t)(kin[j] >> shift) & 0xffu) == (uint32_t)t;
+          for (I j = 0; j < (back + 1) * tkeys; ++j) prev += ((uint32_t)(kin[j] >> shift) & 0xffu) == (uint32_t)t;
           break;
         }
         __nanosleep(64);
@@ -257,7 +261,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
     const uint64_t kv = sk[q];
     const int d = (int)((kv >> shift) & 0xff);
     const uint32_t pos = gbase[d] + (uint32_t)q - lbase[d];
-    if (pos < (uint32_t)n) {  // always, unless calls that share the static scratch overlap
+    if ((I)pos < n) {  // always, unless calls that share the static scratch overlap
       kout[pos] = kv;
       vout[pos] = sv[q];
     }
