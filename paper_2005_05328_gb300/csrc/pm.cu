@@ -715,6 +715,7 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_plane(const cplx<R>* __restri
     }
     const int nb = __shfl_down_sync(0xffffffffu, b, 1);
     if (b > 0 && (lane == 31 || nb != b)) rows[w * nbins + b - 1] += v;
+    __syncwarp();  // the next 32 modes add to the same bins from other lanes
   }
   __syncthreads();
   for (int q = threadIdx.x; q < nbins; q += kPkThreads) {
