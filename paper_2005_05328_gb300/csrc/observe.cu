@@ -182,14 +182,22 @@ __host__ __device__ inline int64_t alm_index(int lmax, int l, int m) {
   return (int64_t)m * (2 * lmax + 1 - m) / 2 + l;
 }
 
-// x^m, m >= 0, by repeated squaring
+// x^m, m >= 0, by repeated squaring in two words: a squaring's rounding would be
+// doubled by every one that follows it (x^256 off by up to 128 of them); a m-fold
+// product, which this replaced, rounds m times
 __device__ __forceinline__ double ipow(double x, int m) {
-  double v = 1.0;
+  double v = 1.0, vl = 0.0, xl = 0.0;
   for (;;) {
-    if (m & 1) v *= x;
+    if (m & 1) {
+      const double p = v * x;
+      vl = fma(v, xl, fma(vl, x, fma(v, x, -p)));
+      v = p;
+    }
     m >>= 1;
-    if (m == 0) return v;
-    x *= x;
+    if (m == 0) return v + vl;
+    const double p = x * x;
+    xl = fma(2.0 * x, xl, fma(x, x, -p));
+    x = p;
   }
 }
 
