@@ -5,8 +5,8 @@ parameter that changes a result stay as given).
 Knobs:
   - walk_eval: how the tree walk evaluates its interaction lists.  The walk has
     one way of evaluating them (two entries at a time, out-of-range ones
-    dropped by a select), which every value selects: results are identical and
-    the candidates' times differ by noise only.
+    dropped by a select), which every value selects: there is nothing to choose,
+    tune_walk times it once for the record and tuned_params runs nothing.
   - host_threads, steps_per_slice of the serving loop (dzs_serve): how many
     host threads issue the mocks' kernels and how many steps each slice
     enqueues.
@@ -22,7 +22,7 @@ import json
 import os
 import time
 
-from . import WALK_GUARDED, WALK_MASKED, Context, dzs_serve, params
+from . import WALK_AUTO, WALK_GUARDED, WALK_MASKED, Context, dzs_serve, params
 
 
 def cache_path() -> str:
@@ -68,35 +68,38 @@ def _walk_ms(p, warm_steps: int, steps: int) -> float:
     return prof["walk"][0] / max(1, done)
 
 
+def _walk_key(n1d, mesh, box, precision, device, physics) -> str:
+    return "walk|%s|n1d=%d|mesh=%d|box=%g|prec=%d|%s" % (_gpu_name(device), n1d, mesh, box, precision,
+                                                      ",".join("%s=%s" % kv for kv in sorted(physics.items())))
+
+
 def tune_walk(n1d: int, mesh: int, box: float, precision: int = 0, device: int = 0, force: bool = False,
               **physics) -> int:
-    """Best walk_eval for this workload shape (cached).  The candidates are
-    timed over a few steps early in the run (near-uniform, where the list
-    evaluation matters most) and a few steps late (clustered)."""
-    key = "walk|%s|n1d=%d|mesh=%d|box=%g|prec=%d|%s" % (_gpu_name(device), n1d, mesh, box, precision,
-                                                     ",".join("%s=%s" % kv for kv in sorted(physics.items())))
+    """walk_eval for this workload shape (cached) with the walk's milliseconds:
+    a few steps early in the run (near-uniform, where the list evaluation matters
+    most) and a few late (clustered).  Every value selects the same evaluation,
+    which is timed once."""
+    key = _walk_key(n1d, mesh, box, precision, device, physics)
     db = _load()
     if not force and key in db:
         return int(db[key]["walk_eval"])
-    base = dict(n1d=n1d, mesh=mesh, box=box, precision=precision, device=device, **physics)
-    nst = params(**base).nsteps
-    timings = {}
-    for mode in (WALK_MASKED, WALK_GUARDED):
-        p = params(**base, walk_eval=mode)
-        timings[mode] = _walk_ms(p, 2, 3) + _walk_ms(p, int(0.8 * nst), 3)
-    best = min(timings, key=timings.get)
-    db[key] = {"walk_eval": int(best), "ms": {str(k): v for k, v in timings.items()}, "when": time.time()}
+    p = params(n1d=n1d, mesh=mesh, box=box, precision=precision, device=device, **physics)
+    ms = _walk_ms(p, 2, 3) + _walk_ms(p, int(0.8 * p.nsteps), 3)
+    db[key] = {"walk_eval": WALK_MASKED, "ms": {str(k): ms for k in (WALK_MASKED, WALK_GUARDED)}, "when": time.time()}
     _store(db)
-    return int(best)
+    return WALK_MASKED
 
 
 def tuned_params(**kw):
-    """params(**kw) with walk_eval chosen by tune_walk (unless given)"""
+    """params(**kw) with walk_eval, unless given, as an earlier tune_walk of this
+    shape cached it, else WALK_AUTO (no run is timed for it)"""
     if "walk_eval" not in kw:
         physics = {k: v for k, v in kw.items() if k not in ("n1d", "mesh", "box", "precision", "device", "seed",
                                                              "sigma8", "lc_capacity", "capacity")}
-        kw = dict(kw, walk_eval=tune_walk(kw["n1d"], kw["mesh"], kw["box"], kw.get("precision", 0),
-                                          kw.get("device", 0), **physics))
+        db = _load()
+        entry = db and db.get(_walk_key(kw["n1d"], kw["mesh"], kw["box"], kw.get("precision", 0),
+                                        kw.get("device", 0), physics))
+        kw = dict(kw, walk_eval=int(entry["walk_eval"]) if entry else WALK_AUTO)
     return params(**kw)
 
 
