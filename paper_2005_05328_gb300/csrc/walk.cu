@@ -54,8 +54,11 @@
 // Queued leaf particles and the COM-first node test: 2.41, 0.57, 33.9 -> 2.30,
 // 0.56, 31.2 ms.  Walking two sibling groups together took 2.58 and 39.5 ms (39%
 // fewer rounds, but the shared list has a third more pairs).
+#include <algorithm>
 #include <cmath>
+#include <exception>
 #include <mutex>
+#include <thread>
 #include <vector>
 
 #include "common.cuh"
@@ -1084,8 +1087,8 @@ void walk_impl(dzs_ctx* c, bool tree, bool close_kick, int step) {
 }
 
 // coefficients of F on each cell of z: Chebyshev interpolation in the cell's
-// own variable, rewritten in powers of z - (cell middle)
-void fill_ztab(double (*tab)[kZDeg + 1]) {
+// own variable, rewritten in powers of z - (cell middle); cells [c0, c1)
+void fill_ztab(double (*tab)[kZDeg + 1], int c0, int c1) {
   typedef long double ld;
   constexpr int n = kZDeg + 1;
   const ld pi = 3.14159265358979323846264338327950288L, tsp = 1.12837916709551257389615890312154517L;
@@ -1102,7 +1105,7 @@ void fill_ztab(double (*tab)[kZDeg + 1]) {
       const ld a = cosl(pi * j * (k + 0.5L) / n) * (j == 0 ? 1.0L : 2.0L) / n;
       for (int p = 0; p <= j; ++p) to_mono[p][k] += cheb[j][p] * a;
     }
-  for (int c = 0; c < kZCells; ++c) {
+  for (int c = c0; c < c1; ++c) {
     const ld width = ldexpl(1.0L / kZSub, kZLo + c / kZSub), half = 0.5L * width;
     const ld mid = ldexpl(1.0L, kZLo + c / kZSub) + width * (c % kZSub) + half;
     ld f[n], mono[n] = {0};
@@ -1115,6 +1118,23 @@ void fill_ztab(double (*tab)[kZDeg + 1]) {
     ld scale = 1.0L;
     for (int p = 0; p < n; ++p, scale /= half) tab[c][p] = (double)(mono[p] * scale);
   }
+}
+
+// the whole table by a few threads: quadruple precision is software on Arm, 15 ms
+// by one thread (first FP64 context of a process 6 -> 21 ms).  A thread that
+// cannot be started leaves its cells to this one.
+void fill_ztab(double (*tab)[kZDeg + 1]) {
+  constexpr int parts = 8, step = (kZCells + parts - 1) / parts;
+  auto fill = [tab](int q) { fill_ztab(tab, q * step, std::min(kZCells, (q + 1) * step)); };
+  std::thread th[parts];
+  int begun = 1;
+  try {
+    for (; begun < parts; ++begun) th[begun] = std::thread(fill, begun);
+  } catch (const std::exception&) {
+  }
+  fill(0);
+  for (int q = begun; q < parts; ++q) fill(q);
+  for (int q = 1; q < begun; ++q) th[q].join();
 }
 
 }  // namespace
