@@ -88,7 +88,7 @@ __host__ __device__ constexpr int ring_pairs(int quarter, bool on_zero) { return
 // (upper sign m = 1 mod 4): 2 or 4 FP64 multiply-adds for eight pixels.  The
 // phasors exp(-i pi q / nphi) come from a table (kTable: half a turn, the other
 // half negated), else from a recurrence.  A warp takes even or odd m only.
-// FP64 is the bound (85% of the unit busy with 3.5 operations per four
+// FP64 is the bound (82% of the unit busy with 3.5 operations per four
 // pixels).  Nside 256, lmax 512: 5.69 ms with 6 operations a pixel, now 0.75 ms.
 template <bool kTable>
 __global__ void __launch_bounds__(kDftThreads) k_ring_dft(const unsigned long long* __restrict__ map, int64_t nside,
@@ -223,10 +223,10 @@ __device__ __forceinline__ double warp_sum8(const double (&v)[8], int lane) {
 // Rings north and south of the equator share |lambda|: lambda_lm(-z) =
 // (-1)^(l+m) lambda_lm(z), so one recursion serves F_N + F_S (l + m even) or
 // F_N - F_S (odd).  FP64-bound: 5 operations per (l, m, ring pair), and a
-// quarter of a shuffle-add with 8 pairs a thread.  lambda_mm is the m-th power
+// quarter of a shuffle-add with 8 pairs a thread (74% of the unit busy).  lambda_mm is the m-th power
 // of the sine times a product the block forms once (it was a loop of m square
 // roots and divisions in every thread: most of the kernel's time).  Nside 256,
-// lmax 512: 8.64 ms, now 1.1 ms.
+// lmax 512: 8.64 ms, now 1.12 ms.
 __global__ void __launch_bounds__(kLegThreads) k_legendre(const double2* __restrict__ F, int64_t nside, int lmax,
                                                           double omega, double2* __restrict__ alm) {
   extern __shared__ double sh[];

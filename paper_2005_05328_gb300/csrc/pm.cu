@@ -611,7 +611,7 @@ void pm_interp(dzs_ctx* c) {
 // sum |k| need no spectrum: k_pk_shells counts the (ky, kz) pairs of each
 // ky^2 + kz^2 once, k_pk_final convolves that with kx^2.  Deterministic.
 // 256^3 particles, mesh 512, 256 bins: 19.7 ms with an FP64 square root,
-// division and 96 FP64 shuffle-adds per 32 modes, now 0.23 + 0.09 ms (planes,
+// division and 96 FP64 shuffle-adds per 32 modes, now 0.24 + 0.09 ms (planes,
 // final; 0.3 GB of the spectrum read, the modes beyond the last bin skipped).
 constexpr int kPkThreads = 256;
 constexpr int pk_split(int M) { return M >= 16 ? 4 : 1; }  // blocks per kx plane
@@ -643,9 +643,9 @@ __device__ __forceinline__ float two_sum(float a, float b, float& s) {
 // words (hi and lo by exact additions; rest collects what those leave, 2^-48 of hi,
 // rounded to 2^-24 of that).  Largest error over random sums 1.6 units of 2^-53, of
 // the FP64 chain 5.2.  That chain, two conversions and two multiply-adds a clock and
-// SM, took 0.22 ms more at mesh 512 (P(k) 4.54 -> 4.76 ms; three words 4.54, two,
-// which keep 48 bits only, 4.53).  Where a remainder may leave the FP32 range the
-// FP64 sum decides.
+// SM, takes 0.22 ms more at mesh 512 (P(k) 4.54 against 4.76 ms; two words, which
+// keep 48 bits only, 4.53; with the weights tabulated three words 4.51).  Where a
+// remainder may leave the FP32 range the FP64 sum decides.
 __device__ __forceinline__ double squares(const cplx<float> (&d)[4]) {
   float hi = 0.f, lo = 0.f, rest = 0.f;
 #pragma unroll
@@ -677,12 +677,15 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_plane(const cplx<R>* __restri
   extern __shared__ double pk_sm[];
   const int H = M / 2 + 1, HP = spec_row<R>(M), kx = blockIdx.x, nw = kPkThreads / 32;
   double* rows = pk_sm;              // [warps][nbins]
-  double* iw = pk_sm + nw * nbins;   // [H] 1 / W_i^2
+  double* wxy = pk_sm + nw * nbins;  // [H] 1 / (W_kx W_ky)^2
+  double* wz = wxy + H;              // [H] modes a half-spectrum point stands for / W_kz^2
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int q = threadIdx.x; q < nw * nbins; q += kPkThreads) rows[q] = 0.0;
+  const double wx = (double)gtab[M + kx], ix = 1.0 / (wx * wx);
   for (int q = threadIdx.x; q < H; q += kPkThreads) {
-    const double wv = (double)gtab[M + q];
-    iw[q] = 1.0 / (wv * wv);
+    const double wv = (double)gtab[M + q], iw = 1.0 / (wv * wv);
+    wxy[q] = ix * iw;
+    wz[q] = q == 0 || 2 * q == M ? iw : 2.0 * iw;
   }
   __syncthreads();
   const int nmax = nbins * nbins + nbins;  // largest |n|^2 of the last bin
@@ -703,7 +706,7 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_plane(const cplx<R>* __restri
       const cplx<R> d[4] = {spec[(px + ky) * HP + kz], twox ? spec[(qx + ky) * HP + kz] : zero,
                             twoy ? spec[(px + M - ky) * HP + kz] : zero,
                             twox && twoy ? spec[(qx + M - ky) * HP + kz] : zero};
-      v = squares(d) * (iw[kx] * iw[ky]) * (kz == 0 || 2 * kz == M ? iw[kz] : 2.0 * iw[kz]);
+      v = squares(d) * wxy[ky] * wz[kz];
     }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -786,7 +789,7 @@ void pk_impl(dzs_ctx* c, int nbins, double* d_part, double* d_out, double shot) 
   unsigned* pairs = (unsigned*)(d_part + (int64_t)nparts * nbins);
   cudaMemsetAsync(pairs, 0, sizeof(unsigned) * (smax + 1), c->stream);
   k_pk_shells<<<grid_for((int64_t)(M / 2 + 1) * (M / 2 + 1)), kThreads, 0, c->stream>>>(M, smax, pairs);
-  const size_t smem = ((size_t)(kPkThreads / 32) * nbins + M / 2 + 1) * sizeof(double);
+  const size_t smem = ((size_t)(kPkThreads / 32) * nbins + 2 * (M / 2 + 1)) * sizeof(double);
   k_pk_plane<R><<<dim3(M / 2 + 1, split), kPkThreads, smem, c->stream>>>(
       (const cplx<R>*)B.spec, M, (const R*)B.green_axis, nbins, d_part);
   k_pk_final<<<nbins, kPkThreads, 0, c->stream>>>(d_part, nparts, pairs, M, nbins, norm, shot, 2.0 * M_PI / L, d_out);
