@@ -19,18 +19,22 @@ namespace {
 constexpr int kSortThreads = 256;
 constexpr int kDigits = 256;
 constexpr int kPasses = 8;
-// Tiles.  Capacity from 2^19 on: 512 threads with 2, 6 or 14 keys each, the
-// smallest of which one wave holds all keys (two blocks per SM of 152; 14 is what
-// the shared memory of two blocks takes).  The count decides, on the device: DZS
-// shrinks the set under a fixed capacity, and tiles of 14 for every count left
-// most SMs without one (sort stage of 66k / 140k / 300k / 541k / 885k keys in a
-// 128^3 context: 171, 191, 204, 210, 215 us; now 91, 104, 124, 143, 156; 2.1M 247,
-// 250, 16.8M 1510, 1490).  Below 2^19: 256 x 4.
+// Tiles.  Capacity from 2^19 on: 512 threads with 2, 6 or 14 keys each (14: what the
+// shared memory of two blocks an SM takes).  The grid holds the capacity in tiles of
+// 14, 152 blocks (one an SM) at least; the count decides on the device, as DZS
+// shrinks the set under a fixed capacity: the smallest tile of which one wave of the
+// grid (two blocks an SM) holds all keys.  Tiles of 14 for every count left most SMs
+// without one: sort stage of 66k / 140k / 300k / 541k / 885k keys in a 128^3 context
+// 171, 191, 204, 210, 215 us, now 91, 104, 124, 143, 156; 2.1M 247, 249, 16.8M 1510,
+// 1490.  A grid of two blocks an SM for 96^3 too, and so 6 keys at 885k, is faster
+// alone (165 -> 155 us) but took 2% off eight mocks stepping together.  Below 2^19:
+// 256 x 4.
 constexpr int kLargeThreads = 512, kLargeItems = 14, kSmallThreads = 256, kSmallItems = 4;
 constexpr int kStep1 = 2, kStep2 = 6;
-constexpr int64_t kLargeFrom = 1 << 19, kWave = 2 * 152;
-__host__ __device__ constexpr int tile_items(int64_t n) {
-  return n <= kWave * kLargeThreads * kStep1 ? kStep1 : n <= kWave * kLargeThreads * kStep2 ? kStep2 : kLargeItems;
+constexpr int64_t kLargeFrom = 1 << 19, kSMs = 152;
+__device__ __forceinline__ int tile_items(int n, int tiles) {
+  const int wave = kLargeThreads * min(tiles, 2 * (int)kSMs);
+  return n <= kStep1 * wave ? kStep1 : n <= kStep2 * wave ? kStep2 : kLargeItems;
 }
 
 // status word of a (tile, digit): count in the low 30 bits, and whether it is
@@ -45,12 +49,11 @@ std::atomic<int> g_look_limit{kLookLimit};
 // tables of status words (a pass fills one and clears the other for the next)
 constexpr int kOffTicket = kPasses * kDigits, kOffStatus = kOffTicket + 32;
 
-// most tiles of any count up to cap: a wave of the smaller tiles, the largest
-// tiles beyond
+// tiles (blocks) of a context: no count up to cap needs more
 inline int64_t sort_tiles(int64_t cap) {
   const int64_t tile = cap >= kLargeFrom ? kLargeThreads * kLargeItems : kSmallThreads * kSmallItems;
   const int64_t full = (cap + tile - 1) / tile;
-  return cap >= kLargeFrom && full < kWave ? kWave : full;
+  return cap >= kLargeFrom && full < kSMs ? kSMs : full;
 }
 // shared memory of a pass: the tile's keys and values, the warps' counters
 constexpr size_t pass_smem(int threads, int items) {
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(kThr, 1024 / kThr)
   if (t == 0) s_tile = (int)atomicAdd(&scratch[kOffTicket + pass], 1u);
   for (int q = t; q < kW * kDigits / 2; q += kThr) reinterpret_cast<uint32_t*>(&wcnt[0][0])[q] = 0;
   __syncthreads();
-  const int items = kVar ? tile_items(n) : kItems;
+  const int items = kVar ? tile_items((int)n, tiles) : kItems;
   const I tkeys = kThr * items;
   const I tile = s_tile, base = tile * tkeys;
   if (tile >= tiles) return;  // never, unless calls that share the static scratch overlap

@@ -1,7 +1,9 @@
 """The radix sort of a large context (capacity from 2^19 on), whose tiles follow
-the count on the device: counts at the edges where a thread takes 2, 6 or 14
-keys (304 blocks of 512 threads in a wave), from one tile to the largest tiles, against the oracle's stable Morton order, exactly; and a count
-that shrinks from call to call in one context, as DZS shrinks it."""
+the count on the device: counts at the edges where a thread takes 2, 6 or 14 keys
+(512 threads a block; waves of 152 blocks in a 96^3 context, of 304 in a 192^3
+one), from one tile to the largest tiles, against the oracle's stable Morton order,
+exactly; and a count that shrinks from call to call in one context, as DZS shrinks
+it."""
 import numpy as np
 import pytest
 
@@ -9,7 +11,7 @@ import oracle as O
 
 pytestmark = pytest.mark.gpu
 
-WAVE = 2 * 152 * 512
+SLOTS = {96: 152, 192: 304}  # blocks of a wave
 
 
 @pytest.fixture(scope="module")
@@ -21,9 +23,9 @@ def dzs():
     return m
 
 
-@pytest.fixture(scope="module")
-def ctx(dzs):
-    with dzs.Context(n1d=192, mesh=96, box=192.0) as c:  # 7.1M slots
+@pytest.fixture(scope="module", params=[96, 192])
+def ctx(dzs, request):
+    with dzs.Context(n1d=request.param, mesh=96, box=2.0 * request.param) as c:
         yield c
 
 
@@ -39,11 +41,16 @@ def check(dzs, ctx, n, pattern):
 
 
 @pytest.mark.parametrize("pattern", ["random", "ties"])
-@pytest.mark.parametrize("n", [14 * WAVE + 1, 14 * WAVE, 6 * WAVE + 1, 6 * WAVE, 6 * WAVE - 1, 2 * WAVE + 1, 2 * WAVE,
-                               2 * WAVE - 1, WAVE + 1, 1025, 1024, 1])
-def test_counts(dzs, ctx, n, pattern):
-    check(dzs, ctx, n, pattern)
+@pytest.mark.parametrize("keys,plus", [(14, 1), (14, 0), (6, 1), (6, 0), (6, -1), (2, 1), (2, 0), (2, -1), (1, 1)])
+def test_counts(dzs, ctx, keys, plus, pattern):
+    n1d = ctx.params.n1d
+    check(dzs, ctx, min(n1d ** 3, keys * 512 * SLOTS[n1d] + plus), pattern)
+
+
+@pytest.mark.parametrize("n", [1, 1024, 1025, 3073])
+def test_few(dzs, ctx, n):
+    check(dzs, ctx, n, "random")
 
 
 def test_full_capacity(dzs, ctx):
-    check(dzs, ctx, 192 ** 3, "random")
+    check(dzs, ctx, ctx.params.n1d ** 3, "random")
