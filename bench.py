@@ -72,8 +72,8 @@ IMPL_BYTES = {
 # of the bench mock, profiles/ncu_k_walk_c2_128cubed_step11.md) and the walk
 # source it was taken on: reported as roofline traffic only while the source
 # is unchanged
-WALK_TRAFFIC_BYTES = 147.683840e6 + 34.484224e6
-WALK_TRAFFIC_SRC = "55ca19b8b1cdc8a4"
+WALK_TRAFFIC_BYTES = 147.097856e6 + 34.066176e6
+WALK_TRAFFIC_SRC = "98ca86d36797fa11"
 
 # serving sample (Poisson stream of mock requests, sizes 32^3 .. 256^3)
 SERVE_RATE = 4.0

@@ -25,7 +25,7 @@ constexpr int kPasses = 8;
 // shrinks the set under a fixed capacity: the smallest tile of which one wave of the
 // grid (two blocks an SM) holds all keys.  Tiles of 14 for every count left most SMs
 // without one: sort stage of 66k / 140k / 300k / 541k / 885k keys in a 128^3 context
-// 171, 191, 204, 210, 215 us, now 91, 104, 124, 143, 156; 2.1M 247, 249, 16.8M 1510,
+// 171, 191, 204, 210, 215 us, now 92, 104, 124, 143, 157; 2.1M 247, 249, 16.8M 1510,
 // 1490.  A grid of two blocks an SM for 96^3 too, and so 6 keys at 885k, is faster
 // alone (165 -> 155 us) but took 2% off eight mocks stepping together.  Below 2^19:
 // 256 x 4.
